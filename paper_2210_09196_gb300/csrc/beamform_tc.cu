@@ -260,7 +260,7 @@ beamform_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
-        if (lane == 0) {
+        if (elect_one()) {
             long long gch = 0;
             bool ok = true;
             const uint64_t pol = l2_policy_evict_first();   // every FFT output tile is read once
@@ -298,7 +298,7 @@ beamform_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t idesc = instr_desc(kTileM, N);
             const uint32_t a_lbo = (uint32_t)g.chunk_rows * 128;   // FP16: between the two 64-subcarrier halves
             long long gch = 0;

@@ -160,7 +160,7 @@ beamform_tf32_kernel(const __grid_constant__ CUtensorMap tmap, Tf32Args g, const
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
-        if (lane == 0) {
+        if (elect_one()) {
             long long gch = 0;
             bool ok = true;
             for (long long i = 0; i < n_my && ok; ++i) {
@@ -187,7 +187,7 @@ beamform_tf32_kernel(const __grid_constant__ CUtensorMap tmap, Tf32Args g, const
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t idesc = idesc_tf32(kTileM, N);
             long long gch = 0;
             bool ok = true;

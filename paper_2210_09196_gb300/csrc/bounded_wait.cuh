@@ -11,6 +11,7 @@ namespace pusch {
 namespace bw {
 
 constexpr uint64_t kWaitNs = 2000000000ull;  // the library kernels' limit: 2 s
+constexpr int kPollsPerTimer = 64;           // polls between two reads of the timer
 
 __device__ __forceinline__ uint64_t globaltimer() {
     uint64_t t;
@@ -37,11 +38,14 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
 // Waits until the phase with the given parity of the barrier at shared address `bar` has completed, for at
 // most limit_ns nanoseconds of %globaltimer. Returns false when the limit passed first.
 __device__ __forceinline__ bool mbar_wait_for(uint32_t bar, uint32_t parity, uint64_t limit_ns) {
-    if (mbar_try_wait(bar, parity)) return true;
+    for (int k = 0; k < kPollsPerTimer; ++k)
+        if (mbar_try_wait(bar, parity)) return true;
     const uint64_t deadline = globaltimer() + limit_ns;
-    while (!mbar_try_wait(bar, parity))
+    for (;;) {
+        for (int k = 0; k < kPollsPerTimer; ++k)
+            if (mbar_try_wait(bar, parity)) return true;
         if (globaltimer() > deadline) return false;
-    return true;
+    }
 }
 
 }  // namespace bw

@@ -112,7 +112,7 @@ conv32_tc_kernel(const __grid_constant__ CUtensorMap tin, ConvTcArgs g, const __
 
     if (warp == 0) {
         // ---------------------------------------------------------------- TMA producer
-        if (lane == 0) {
+        if (elect_one()) {
             long long i = 0;
             for (; i < n_my; ++i) {
                 const int s = (int)(i % kStages);
@@ -137,7 +137,7 @@ conv32_tc_kernel(const __grid_constant__ CUtensorMap tin, ConvTcArgs g, const __
         }
     } else if (warp == 1) {
         // ---------------------------------------------------------------- MMA issuer
-        if (lane == 0) {
+        if (elect_one()) {
             for (long long i = 0; i < n_my; ++i) {
                 const int s = (int)(i % kStages), buf = (int)(i & 1);
                 if (!mbar_wait(smem_u32(&sh.tempty[buf]), (uint32_t)(((i >> 1) & 1) ^ 1), abort, err)) break;

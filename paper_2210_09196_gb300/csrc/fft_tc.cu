@@ -144,7 +144,7 @@ fft_tc_kernel(const __grid_constant__ CUtensorMap tin, __half *__restrict__ out,
 
     if (warp == kEpiWarps) {
         // ------------------------------------------------------------ control: row copies and MMAs
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t idesc = idesc_f16(128, 128, true, false);   // A MN-major in both stages
             // the time samples are read once: evict-first, so that they do not push the FFT output (the next
             // kernel's input) out of L2 (an evict-last hint on the 2-byte output stores measured slower)

@@ -18,6 +18,7 @@ using bw::globaltimer;
 using bw::mbar_init;
 using bw::mbar_try_wait;
 constexpr uint64_t kWaitNs = bw::kWaitNs;  // 2 s
+using bw::kPollsPerTimer;
 
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
@@ -27,12 +28,31 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
+// True in one lane of the converged warp. Work that one thread does with tensor-core or copy instructions goes
+// under this predicate, not under lane == 0: those instructions take their operands from uniform registers, and
+// only under elect.sync does the compiler know that one lane is active; under lane == 0 it loops over the lanes for
+// each of them (194 clocks per tcgen05.mma against 40 to 64, the operands' shared-memory reads, in a loop of MMAs
+// alone on GB300).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(p));
+    return p != 0;
+}
+
 // Bounded wait on an mbarrier phase. Gives up when the deadline passes (sets *abort and the error bit) or
-// when another role has already aborted; returns false then.
+// when another role has already aborted; returns false then. The timer is read once in kPollsPerTimer polls: a
+// read of %globaltimer takes far longer than a poll, and one in every poll delayed each hand-over by as much.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *abort, uint32_t *err) {
-    if (mbar_try_wait(bar, parity)) return true;
+    for (int k = 0; k < kPollsPerTimer; ++k)
+        if (mbar_try_wait(bar, parity)) return true;
     const uint64_t deadline = globaltimer() + kWaitNs;
-    while (!mbar_try_wait(bar, parity)) {
+    for (;;) {
+        for (int k = 0; k < kPollsPerTimer; ++k)
+            if (mbar_try_wait(bar, parity)) return true;
         if (*abort) return false;
         if (globaltimer() > deadline) {
             *abort = 1;
@@ -40,25 +60,29 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
             return false;
         }
     }
-    return true;
 }
 
 // mbar_wait with a pause of about `sleep_ns` between polls, for waits that usually last a while (another role's
 // work): the polling lane then leaves the issue slots to the warps that do that work.
 __device__ __forceinline__ bool mbar_wait_sleep(uint32_t bar, uint32_t parity, volatile int *abort, uint32_t *err,
                                                 unsigned sleep_ns) {
-    if (mbar_try_wait(bar, parity)) return true;
+    for (int k = 0; k < kPollsPerTimer; ++k) {
+        if (mbar_try_wait(bar, parity)) return true;
+        __nanosleep(sleep_ns);
+    }
     const uint64_t deadline = globaltimer() + kWaitNs;
-    while (!mbar_try_wait(bar, parity)) {
+    for (;;) {
+        for (int k = 0; k < kPollsPerTimer; ++k) {
+            if (mbar_try_wait(bar, parity)) return true;
+            __nanosleep(sleep_ns);
+        }
         if (*abort) return false;
         if (globaltimer() > deadline) {
             *abort = 1;
             if (err) atomicOr(err, kErrTensorWait);
             return false;
         }
-        __nanosleep(sleep_ns);
     }
-    return true;
 }
 
 // Wait used while draining after an abort: bounded, ignores the abort flag.
