@@ -203,6 +203,7 @@ KERNELS = {"fft": {"tc": ("fft_tc_kernel", "fft_tc.cu+" + TC), "simt": ("fft_ker
            "beamform": {"mixed": ("beamform_tc_kernel", "beamform_tc.cu+" + TC),
                         "fp8": ("beamform_tc_kernel", "beamform_tc.cu+" + TC),
                         "fp32": ("beamform_tf32_kernel", "beamform_tf32.cu+" + TC),
+                        "fp32_k": ("beamform_tf32k_kernel", "beamform_tf32k.cu+" + TC),
                         "fp32_simt": ("beamform_fp32_kernel", "beamform.cu")},
            "ls": ("ls_pilots_kernel", "chest.cu+chest_common.cuh"),
            "detect": ("mmse_kernel", "mmse_impl.cuh+detect_core.cuh+detect_tc.cuh+chest_common.cuh")}
@@ -218,7 +219,8 @@ def kernel_of(stage, form, cell=None):
     if stage == "beamform" and form == "fp32" and cell is not None and not (
             cell.n_sc % 2 == 0 and cell.n_rx % 16 == 0 and cell.n_beams % 8 == 0 and cell.n_beams <= 64
             and 32 * cell.n_rx * cell.n_beams <= 96 * 1024):
-        return k["fp32_simt"]                    # the FP32 form's 3xTF32 tensor-core GEMM needs these shapes
+        # the whole of W does not fit one CTA: the antennas are split over a cluster, or FP32 FMAs
+        return k["fp32_k" if 32 <= cell.n_rx <= 256 and cell.n_beams > 32 else "fp32_simt"]
     return k[form] if isinstance(k, dict) else k
 
 
