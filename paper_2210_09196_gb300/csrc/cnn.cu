@@ -277,32 +277,11 @@ int param_offset(int layer) {
 
 int cnn_param_count() { return param_offset(4); }
 
-// Forward pass of n grids of width w. acts: [3][n][32][2][ld] bf16 (post-ReLU activations, rows of ld >= w
-// elements), x: [n][2][2][w] bf16, y: [n][2][2][w] f32. The two 32 -> 32 layers run on the tensor cores
-// (cnn_tc.cu) when ld is a multiple of 8 (16-byte rows for the copy engine), on the FP32 pipes otherwise.
+// Forward pass of n grids of width w (cnn_tc.cu). x: [n][2][2][w] bf16, y: [n][2][2][w] f32; acts (or NULL):
+// [3][n][32][2][w] bf16, the post-ReLU activations.
 cudaError_t cnn_forward(int n, int w, const __nv_bfloat16 *x, const __nv_bfloat16 *P, float *y, __nv_bfloat16 *acts,
-                        cudaStream_t st, int ld, uint32_t *err) {
-    if (ld <= 0) ld = w;
-    const size_t big = (size_t)n * 32 * 2 * ld;
-    const __nv_bfloat16 *W0 = P + param_offset(0), *W1 = P + param_offset(1), *W2 = P + param_offset(2),
-                        *W3 = P + param_offset(3);
-    cudaError_t e;
-    if ((e = launch_conv<2, 32, __nv_bfloat16, kOutReluBf16>(x, W0, W0 + 32 * 2 * 9, acts, nullptr, n, w, kDil[0],
-                                                             st, w, ld)) != cudaSuccess)
-        return e;
-    for (int k = 1; k <= 2; ++k) {
-        const __nv_bfloat16 *Wk = k == 1 ? W1 : W2;
-        const __nv_bfloat16 *in = acts + (k - 1) * big;
-        __nv_bfloat16 *out = acts + k * big;
-        if (conv32_tc_supported(ld, kDil[k]))
-            e = launch_conv32_tc(in, Wk, Wk + 32 * 32 * 9, out, n, w, ld, kDil[k], err, st);
-        else
-            e = launch_conv<32, 32, __nv_bfloat16, kOutReluBf16>(in, Wk, Wk + 32 * 32 * 9, out, nullptr, n, w, kDil[k],
-                                                                 st, ld, ld);
-        if (e != cudaSuccess) return e;
-    }
-    return launch_conv<32, 2, __nv_bfloat16, kOutResidF32>(acts + 2 * big, W3, W3 + 2 * 32 * 9, y, x, n, w, kDil[3],
-                                                           st, ld, w);
+                        cudaStream_t st, uint32_t *err) {
+    return launch_cnn_fwd(x, P, y, acts, n, w, err, st);
 }
 
 // Backward pass: grad (zeroed here) = d mean((y - target)^2) / d params; *loss = that mean (if loss != NULL).
