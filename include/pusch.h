@@ -298,7 +298,7 @@ pusch_status pusch_cnn_forward(int n, int w, const void *x_bf16, const void *par
 
 /* grad (FP32, param_count values, overwritten) = d/dparams of mean((y - target)^2) for the forward pass
  * that produced y and acts; *loss (if not NULL) = that mean. work: 2 * n * 32 * 2 * w floats of scratch;
- * wflip: param_count bf16 values of scratch. */
+ * wflip: param_count bf16 values of scratch (not used any more). */
 pusch_status pusch_cnn_backward(int n, int w, const void *x_bf16, const void *acts_bf16, const void *params_bf16,
                                 const float *y, const float *target, float *grad, float *loss, float *work,
                                 void *wflip_bf16, void *stream);

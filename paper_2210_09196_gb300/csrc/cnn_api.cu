@@ -49,7 +49,7 @@ pusch_status pusch_cnn_backward(int n, int w, const void *x, const void *acts, c
         return cfail(PUSCH_ERR_ARG, "pusch_cnn_backward: NULL buffer");
     cudaError_t e = pusch::cnn_backward(n, w, (const __nv_bfloat16 *)x, (const __nv_bfloat16 *)acts,
                                         (const __nv_bfloat16 *)params, y, target, grad, loss, work,
-                                        (__nv_bfloat16 *)wflip, (cudaStream_t)stream);
+                                        (cudaStream_t)stream);
     if (e != cudaSuccess) return cfail(PUSCH_ERR_CUDA, "CNN backward launch", e);
     pusch::set_last_error("");
     return PUSCH_OK;

@@ -220,8 +220,10 @@ cudaError_t cnn_forward(int n, int w, const __nv_bfloat16 *x, const __nv_bfloat1
 cudaError_t launch_cnn_fwd(const __nv_bfloat16 *in, const __nv_bfloat16 *P, float *y, __nv_bfloat16 *acts, int n, int w,
                            uint32_t *err, cudaStream_t st);
 cudaError_t cnn_backward(int n, int w, const __nv_bfloat16 *x, const __nv_bfloat16 *acts, const __nv_bfloat16 *P,
-                         const float *y, const float *target, float *grad, float *loss, float *work,
-                         __nv_bfloat16 *wflip, cudaStream_t st);
+                         const float *y, const float *target, float *grad, float *loss, float *work, cudaStream_t st);
+cudaError_t launch_cnn_bwd(int n, int w, const __nv_bfloat16 *x, const __nv_bfloat16 *acts, const __nv_bfloat16 *P,
+                           const float *y, const float *target, float *grad, float *loss, float *work, uint32_t *err,
+                           cudaStream_t st);
 cudaError_t cnn_adam(int step, float lr, float b1, float b2, float eps, float *p, __nv_bfloat16 *pb, const float *g,
                      float *m, float *v, cudaStream_t st);
 cudaError_t launch_ls_grid(const Geometry &g, int n_slots, const float2 *beam, const float2 *pilots,
