@@ -123,9 +123,7 @@ __device__ __forceinline__ bool factor_solve_rhs_lanes(float2 (&G)[NL], float2 *
                 dj = 1.f;
             }
             const float inv = rsqrtf(dj);
-            if (i > j) G[j] = cscale(sj, inv);
-            else if (i == j) G[j] = make_float2(dj * inv, 0.f);
-            else G[j] = make_float2(0.f, 0.f);
+            G[j] = cscale(sj, inv);     // lanes i <= j: not read again (their later sums are not used)
             if (i == j) dinv = inv;
             Lrot[j] = make_float2(-G[j].y, G[j].x);
             if (i > j) L4[i * (i - 1) / 2 + j] = make_float4(-G[j].x, -G[j].x, G[j].y, G[j].y);

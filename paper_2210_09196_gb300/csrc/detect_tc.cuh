@@ -4,11 +4,19 @@
 // the M = 16 of this instruction shape exactly (the 5th-generation tcgen05 products start at M = 64, where one
 // subcarrier would fill an eighth of the tile).
 //
-// Real embedding, K along the interleaved (re, im) floats of a row, k = 2 b + c:
-//   A[i][k]   = H[i][b].c                                 (the estimate tile as it sits in shared memory)
-//   Re G = A A^T                                          (B = A^T: the A fragments serve as B fragments)
-//   Im G = A R^T,  R[j][2 b] = Im H[j][b], R[j][2 b + 1] = -Re H[j][b]     (Im(conj(h_i) h_j))
-//   Re r_d = A y_d,  Im r_d = A rot(y_d)                  (the 12 data symbols' re and im parts as 24 columns)
+// The real and imaginary parts of eight beams are two K = 8 steps (16-byte loads bring two beams' both parts):
+//   Re G = A_r A_r^T + A_i A_i^T                          (B = A^T: the A fragments serve as B fragments)
+//   Im G = X - X^T,  X = A_r A_i^T                        (Im(conj(h_i) h_j); the difference is taken when a lane reads
+//                                                          its row of G from shared memory)
+//   P = A_r Y, Q = A_i Y,  Y = the 12 data symbols' re and im parts as 24 columns;  Re r_d = P[re d] + Q[im d],
+//   Im r_d = P[im d] - Q[re d]
+// Each of the five sums has its own accumulator: the tensor core truncates as it accumulates, which shrinks a sum by an
+// amount that goes with its number of steps, and equal shrinking of G and r_d cancels in x (with Re G in one accumulator
+// of twice the steps x was off by 1.8e-6 instead of 8.6e-7 for 32 layers; the interleaved embedding: 1.3e-6).
+// Against the interleaved embedding (K = 2 N_B, Im G and Im r_d from rotated copies of the operands) this loads and
+// splits each element once instead of twice and takes 36 products per 8 beams instead of 42 (16 layers; 32 layers, with
+// the tiles of Re G above the diagonal left out: 96 instead of 132). Measured on GB300 (pusch_mmse_detect): 16 layers,
+// 32 beams, 8 slots 120 -> 110 us; 32 layers, 64 beams, 2 slots 167 -> 153 us.
 // FP32 accuracy from TF32 operands: every operand x is split into hi = x rounded to TF32 (10 explicit mantissa
 // bits, ties away from zero, by an integer add and mask) and lo = x - hi (exact, |lo| <= 2^-11 |x|), which the
 // tensor core reads truncated to TF32 (|x - hi - lo_tf32| <= 2^-21 |x|); each product is hi*hi + hi*lo + lo*hi
@@ -41,86 +49,81 @@ __device__ __forceinline__ void mma3_tf32(float (&c)[4], const uint32_t (&ah)[4]
 }
 
 // G and r_d (12 data symbols) of one subcarrier by the whole warp.
-//   hf: the subcarrier's estimate rows as floats (row i at hf + i hsf, NL rows, 2 NB floats used)
-//   yf: its data-symbol rows as floats (row d at yf + d ysf), overwritten by r_d: r_d[i] at float2 (d ys + i)
-//   Gs: G[i][j] (float2) at Gs + i (NL + 2) + j, over the estimate rows (written after every lane has read them)
+//   H: the subcarrier's estimate rows (row i at H + i hs, NL rows of nb values)
+//   Y: its data-symbol rows (row d at Y + d ys), overwritten by r_d: r_d[i] at Y[d ys + i]
+//   Gs: (Re G[i][j] for j <= i, X[i][j]) at Gs + i (NL + 2) + j, over the estimate rows (written after every lane has
+//       read them)
 // Fragment layout of m16n8k8 (g = lane / 4, t = lane % 4): A rows g, g + 8 at columns t, t + 4; B column g at
 // rows t, t + 4; the accumulator rows g, g + 8 at columns 2 t, 2 t + 1.
-// NB = 0: the beam count nb at run time (a multiple of 4: K = 2 nb floats in steps of 8).
+// NB = 0: the beam count nb at run time (a multiple of 4; the rest of a last step of 4 beams is zero).
 template <int NL, int NB>
-__device__ __forceinline__ void gram_rhs_tc(const float *hf, int hsf, float *yf, int ysf, int ys, float2 *Gs, int lane,
-                                            int nb = NB) {
+__device__ __forceinline__ void gram_rhs_tc(const float2 *H, int hs, float2 *Y, int ys, float2 *Gs, int lane, int nb = NB) {
     constexpr int MT = NL / 16;     // 16-row tiles of layers
-    constexpr int NG = NL / 8;      // 8-column tiles of G's columns (each for Re and for Im)
+    constexpr int NG = NL / 8;      // 8-column tiles of G's columns
     constexpr int GS = NL + 2;      // row stride of Gs (float2): the 16-byte row loads below spread over banks
-    const int g = lane >> 2, t = lane & 3, to = t ^ 1;
-    const float sg = (t & 1) ? -1.f : 1.f;  // the rotation's sign at column k0 + t (the parity of t)
-    // right-hand-side columns of this lane's B fragments: tile 0 Re r_0..7; tile 1 Re r_8..11 (g < 4) or
-    // Im r_0..3; tile 2 Im r_4..11
-    const int d0 = g, d1 = g < 4 ? 8 + g : g - 4, d2 = 4 + g;
-    const bool rot1 = g >= 4;
-    float cg[MT][2 * NG][4], cr[MT][3][4];
+    const int g = lane >> 2, t = lane & 3;
+    float cg[MT][NG][4], ci[MT][NG][4], cx[MT][NG][4], cp[MT][3][4], cq[MT][3][4];
 #pragma unroll
     for (int m = 0; m < MT; ++m) {
 #pragma unroll
-        for (int n = 0; n < 2 * NG; ++n)
+        for (int n = 0; n < NG; ++n)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) cg[m][n][e] = 0.f;
+            for (int e = 0; e < 4; ++e) cg[m][n][e] = ci[m][n][e] = cx[m][n][e] = 0.f;
 #pragma unroll
         for (int q = 0; q < 3; ++q)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) cr[m][q][e] = 0.f;
+            for (int e = 0; e < 4; ++e) cp[m][q][e] = cq[m][q][e] = 0.f;
     }
-    constexpr int kUnroll = NL == 16 ? 2 : 1;   // two K steps in flight for 16 layers (measured faster; not for 32)
-#pragma unroll kUnroll
-    for (int k0 = 0; k0 < 2 * (NB > 0 ? NB : nb); k0 += 8) {
-        uint32_t ah[MT][4], al[MT][4];
+    // K index t is beam k0 + 2 t, t + 4 is beam k0 + 2 t + 1 (the order of K is free): one 16-byte load brings both
+    const float2 *h0 = H + g * hs + 2 * t;
+    const float2 *y0 = Y + g * ys + 2 * t, *y1 = Y + (8 + (g & 3)) * ys + 2 * t;   // columns g; 8 + g % 4 (re for g < 4, else im)
+    const int n_b = NB > 0 ? NB : nb;
+#pragma unroll 1
+    for (int k0 = 0; k0 < n_b; k0 += 8) {
+        const bool on = NB > 0 || k0 + 2 * t < n_b;
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+        uint32_t rh[MT][4], rl[MT][4], ih[MT][4], il[MT][4];
 #pragma unroll
-        for (int m = 0; m < MT; ++m) {
-            const float *r0 = hf + (16 * m + g) * hsf + k0, *r1 = r0 + 8 * hsf;
-            tf32_split(r0[t], ah[m][0], al[m][0]);
-            tf32_split(r1[t], ah[m][1], al[m][1]);
-            tf32_split(r0[t + 4], ah[m][2], al[m][2]);
-            tf32_split(r1[t + 4], ah[m][3], al[m][3]);
-        }
-        // Re G: B column tile n = rows 8 n .. 8 n + 7 of A, i.e. registers (0, 2) or (1, 3) of A tile n / 2
+        for (int m = 0; m < MT; ++m)
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const float4 v = on ? *reinterpret_cast<const float4 *>(h0 + (16 * m + 8 * q) * hs + k0) : zero;
+                tf32_split(v.x, rh[m][q], rl[m][q]);
+                tf32_split(v.y, ih[m][q], il[m][q]);
+                tf32_split(v.z, rh[m][q + 2], rl[m][q + 2]);
+                tf32_split(v.w, ih[m][q + 2], il[m][q + 2]);
+            }
+        // B column tile n = rows 8 n .. 8 n + 7 of A, i.e. registers (0, 2) or (1, 3) of A tile n / 2
 #pragma unroll
         for (int n = 0; n < NG; ++n) {
             const int mb = n >> 1, j0 = n & 1, j1 = j0 + 2;
 #pragma unroll
-            for (int m = 0; m < MT; ++m)
-                mma3_tf32(cg[m][n], ah[m], al[m], ah[mb][j0], ah[mb][j1], al[mb][j0], al[mb][j1]);
+            for (int m = 0; m < MT; ++m) {
+                if (mb <= m) {
+                    mma3_tf32(cg[m][n], rh[m], rl[m], rh[mb][j0], rh[mb][j1], rl[mb][j0], rl[mb][j1]);
+                    mma3_tf32(ci[m][n], ih[m], il[m], ih[mb][j0], ih[mb][j1], il[mb][j0], il[mb][j1]);
+                }
+                mma3_tf32(cx[m][n], rh[m], rl[m], ih[mb][j0], ih[mb][j1], il[mb][j0], il[mb][j1]);
+            }
         }
-        // Im G: B column tile n = the rotated rows 8 n .. 8 n + 7
-#pragma unroll
-        for (int n = 0; n < NG; ++n) {
-            const float *rr = hf + (8 * n + g) * hsf + k0;
-            uint32_t bh0, bl0, bh1, bl1;
-            tf32_split(sg * rr[to], bh0, bl0);
-            tf32_split(sg * rr[to + 4], bh1, bl1);
-#pragma unroll
-            for (int m = 0; m < MT; ++m) mma3_tf32(cg[m][NG + n], ah[m], al[m], bh0, bh1, bl0, bl1);
-        }
-        // right-hand sides: 24 columns in three tiles
+        // right-hand sides: columns Re y_0..7; Im y_0..7; Re y_8..11 and Im y_8..11
         {
-            uint32_t bh0, bl0, bh1, bl1;
-            const float *y0 = yf + d0 * ysf + k0;
-            tf32_split(y0[t], bh0, bl0);
-            tf32_split(y0[t + 4], bh1, bl1);
+            const float4 va = on ? *reinterpret_cast<const float4 *>(y0 + k0) : zero;
+            const float4 vb = on ? *reinterpret_cast<const float4 *>(y1 + k0) : zero;
+            uint32_t bh[3][2], bl[3][2];
+            tf32_split(va.x, bh[0][0], bl[0][0]);
+            tf32_split(va.z, bh[0][1], bl[0][1]);
+            tf32_split(va.y, bh[1][0], bl[1][0]);
+            tf32_split(va.w, bh[1][1], bl[1][1]);
+            tf32_split(g < 4 ? vb.x : vb.y, bh[2][0], bl[2][0]);
+            tf32_split(g < 4 ? vb.z : vb.w, bh[2][1], bl[2][1]);
 #pragma unroll
-            for (int m = 0; m < MT; ++m) mma3_tf32(cr[m][0], ah[m], al[m], bh0, bh1, bl0, bl1);
-            const float *y1 = yf + d1 * ysf + k0;
-            const int c1 = rot1 ? to : t;
-            const float s1 = rot1 ? sg : 1.f;
-            tf32_split(s1 * y1[c1], bh0, bl0);
-            tf32_split(s1 * y1[c1 + 4], bh1, bl1);
+            for (int q = 0; q < 3; ++q)
 #pragma unroll
-            for (int m = 0; m < MT; ++m) mma3_tf32(cr[m][1], ah[m], al[m], bh0, bh1, bl0, bl1);
-            const float *y2 = yf + d2 * ysf + k0;
-            tf32_split(sg * y2[to], bh0, bl0);
-            tf32_split(sg * y2[to + 4], bh1, bl1);
-#pragma unroll
-            for (int m = 0; m < MT; ++m) mma3_tf32(cr[m][2], ah[m], al[m], bh0, bh1, bl0, bl1);
+                for (int m = 0; m < MT; ++m) {
+                    mma3_tf32(cp[m][q], rh[m], rl[m], bh[q][0], bh[q][1], bl[q][0], bl[q][1]);
+                    mma3_tf32(cq[m][q], ih[m], il[m], bh[q][0], bh[q][1], bl[q][0], bl[q][1]);
+                }
         }
     }
     __syncwarp();  // every lane has read the estimate and data-symbol rows
@@ -129,19 +132,19 @@ __device__ __forceinline__ void gram_rhs_tc(const float *hf, int hsf, float *yf,
 #pragma unroll
         for (int n = 0; n < NG; ++n) {
             const int i = 16 * m + g, j = 8 * n + 2 * t;
-            *reinterpret_cast<float4 *>(Gs + i * GS + j) =
-                make_float4(cg[m][n][0], cg[m][NG + n][0], cg[m][n][1], cg[m][NG + n][1]);
+            *reinterpret_cast<float4 *>(Gs + i * GS + j) = make_float4(
+                cg[m][n][0] + ci[m][n][0], cx[m][n][0], cg[m][n][1] + ci[m][n][1], cx[m][n][1]);
             *reinterpret_cast<float4 *>(Gs + (i + 8) * GS + j) =
-                make_float4(cg[m][n][2], cg[m][NG + n][2], cg[m][n][3], cg[m][NG + n][3]);
+                make_float4(cg[m][n][2] + ci[m][n][2], cx[m][n][2], cg[m][n][3] + ci[m][n][3], cx[m][n][3]);
         }
 #pragma unroll
-        for (int q = 0; q < 3; ++q)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int c = 8 * q + 2 * t + (e & 1), i = 16 * m + g + 8 * (e >> 1);
-                const int d = c < 12 ? c : c - 12;
-                yf[2 * (d * ys + i) + (c < 12 ? 0 : 1)] = cr[m][q][e];
-            }
+        for (int e = 0; e < 4; ++e) {
+            const int c = 2 * t + (e & 1), i = 16 * m + g + 8 * (e >> 1);
+            Y[c * ys + i] = make_float2(cp[m][0][e] + cq[m][1][e], cp[m][1][e] - cq[m][0][e]);
+            // third tile: Re parts in the lanes t < 2, Im parts in t >= 2; the other product is two lanes away
+            const float o = __shfl_xor_sync(kDetFull, cq[m][2][e], 2);
+            reinterpret_cast<float *>(Y + (8 + (c & 3)) * ys + i)[t >> 1] = t < 2 ? cp[m][2][e] + o : cp[m][2][e] - o;
+        }
     }
 }
 
@@ -160,17 +163,18 @@ __device__ __forceinline__ bool detect_group_tc(float2 *Hw, int ht, int hs, floa
     constexpr int SPW = 32 / NL, GS = NL + 2;
 #pragma unroll 1
     for (int gg = 0; gg < SPW; ++gg)
-        gram_rhs_tc<NL, NB>(reinterpret_cast<const float *>(Hw + gg * ht), 2 * hs,
-                            reinterpret_cast<float *>(Yw + gg * 12 * ys), 2 * ys, ys, Hw + gg * ht, lane, nb);
+        gram_rhs_tc<NL, NB>(Hw + gg * ht, hs, Yw + gg * 12 * ys, ys, Hw + gg * ht, lane, nb);
     __syncwarp();
     float2 G[NL];
     {
+        // own row, and the column of X that makes Im G[i][j] = X[i][j] - X[j][i]
         const float4 *row = reinterpret_cast<const float4 *>(Hw + grp * ht + i * GS);
+        const float2 *col = Hw + grp * ht + i;
 #pragma unroll
         for (int j = 0; j < NL / 2; ++j) {
             const float4 v = row[j];
-            G[2 * j] = make_float2(v.x, v.y);
-            G[2 * j + 1] = make_float2(v.z, v.w);
+            G[2 * j] = make_float2(v.x, v.y - col[2 * j * GS].y);
+            G[2 * j + 1] = make_float2(v.z, v.w - col[(2 * j + 1) * GS].y);
         }
     }
     if (sigma2) load += __ldg(&sigma2[slot]);
