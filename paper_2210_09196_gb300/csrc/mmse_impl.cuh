@@ -56,6 +56,19 @@ __device__ __forceinline__ int data_symbol(const MmseArgs &g, int d) {
     return s;
 }
 
+// Slot and subcarrier of the running index sc = slot * n_sc + a. 32-bit where the launch's indexes allow it: a 64-bit
+// division takes some 80 instructions, and a warp needs four (of 4.7 k in all for 16 layers).
+__device__ __forceinline__ void slot_of(long long sc, int n_sc, long long total_sc, long long &slot, int &a) {
+    if (total_sc <= 0x7fffffffLL) {
+        const unsigned q = (unsigned)sc / (unsigned)n_sc;
+        slot = q;
+        a = (int)((unsigned)sc - q * (unsigned)n_sc);
+    } else {
+        slot = sc / n_sc;
+        a = (int)(sc - slot * n_sc);
+    }
+}
+
 // The estimate rows of the warp's SPW subcarriers (from Hq, one group's estimate) -> the warp's H tile, rows
 // padded to stride hs; 16-byte cp.async pieces (two beams) when the beam count is even, 8-byte pieces
 // otherwise; rows of absent layers and subcarriers are zeroed. Waits for all of the lane's copies.
@@ -105,25 +118,31 @@ __device__ __forceinline__ void stage_H_interp(float2 *Ht, const MmseArgs &g, lo
     constexpr int kRows = 32 / kU;        // rows per warp pass (2 for 32 beams, 1 for 64)
     constexpr int kHs = (NB + 3) & ~1;    // row_stride(NB)
     constexpr int kB = 4;                 // passes whose loads are issued together
-    long long base = -1;                  // table row of (slot, layer, k = 0), in 16-byte pieces
-    int klo = 0, khi = 0;
+    // table rows of the bracket, in 16-byte pieces from the table of the warp's first slot (at most two slots away:
+    // 2 * 32 layers * 4096 pilots * 32 pieces fit 32 bits); -1: a row of zeros
+    int olo = -1, ohi = 0;
+    long long sl0;
+    int a00;
+    slot_of(sc0, g.n_sc, total_sc, sl0, a00);
     float w = 0.f;
     {
         const int gg = lane / NL, l = lane - gg * NL;
         const long long sc = sc0 + gg;
         if (l < g.n_layers && sc < total_sc) {
-            const long long sl = sc / g.n_sc;
-            const int a = (int)(sc - sl * g.n_sc), p = g.port[l];
+            long long sl;
+            int a;
+            slot_of(sc, g.n_sc, total_sc, sl, a);
+            const int p = g.port[l];
             int lo, hi;
             pilot_bracket(a, p, g.comb, g.n_sc, lo, hi);
-            klo = (lo - p) / g.comb;
-            khi = (hi - p) / g.comb;
+            const int klo = (lo - p) / g.comb;
+            olo = (((int)(sl - sl0) * g.n_layers + l) * g.kmax + klo) * kU;
+            ohi = hi == lo ? olo : olo + kU;
             w = interp_weight(a, lo, hi);
-            base = (sl * g.n_layers + l) * (long long)g.kmax * kU;
         }
     }
-    const float4 *tab = reinterpret_cast<const float4 *>(g.ls);
     const int sub = lane / kU, u = lane - sub * kU;
+    const float4 *tab = reinterpret_cast<const float4 *>(g.ls) + sl0 * g.n_layers * (long long)g.kmax * kU + u;
     // rows of pass t: when a pass covers SPW rows, the same layer of the warp's SPW subcarriers (neighbouring
     // subcarriers mostly share the bracket, so the pass reads each table line once); else kRows consecutive rows
     constexpr int SPW = 32 / NL;
@@ -136,14 +155,13 @@ __device__ __forceinline__ void stage_H_interp(float2 *Ht, const MmseArgs &g, lo
 #pragma unroll
         for (int q = 0; q < kB; ++q) {
             const int r = row_of(t0 + q);
-            const long long b = __shfl_sync(kFull, base, r);
-            const int kl = __shfl_sync(kFull, klo, r), kh = __shfl_sync(kFull, khi, r);
+            const int ol = __shfl_sync(kFull, olo, r), oh = __shfl_sync(kFull, ohi, r);
             wr[q] = __shfl_sync(kFull, w, r);
-            on[q] = b >= 0;
+            on[q] = ol >= 0;
             lo4[q] = hi4[q] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (on[q]) {
-                lo4[q] = __ldg(tab + b + (long long)kl * kU + u);
-                hi4[q] = __ldg(tab + b + (long long)kh * kU + u);
+                lo4[q] = __ldg(tab + ol);
+                hi4[q] = __ldg(tab + oh);
             }
         }
 #pragma unroll
@@ -160,12 +178,13 @@ __device__ __forceinline__ void stage_H_interp(float2 *Ht, const MmseArgs &g, lo
     }
 }
 
-// Warps per CTA of the 12-data-symbol kernels when not tuned: one (each warp then starts and ends on its own;
-// larger CTAs measured slower for 16 layers, their warps waiting for one another at the output rows), four for
-// 32 layers (one subcarrier per warp).
+// Warps per CTA of the 12-data-symbol kernels when not tuned: one for the small classes (each warp starts and ends on
+// its own); two for 16 layers, whose four subcarriers make a whole 32-byte sector of every x-hat row (16 deployment
+// slots in the chain: one warp 427 us, two 421, four 431, the warps of larger CTAs waiting for one another at the output
+// rows); four for 32 layers (one subcarrier per warp; 2 massive slots: 168 us with one warp, 157, 152, 182 with eight).
 template <int NL>
 constexpr int mmse_default_warps() {
-    return NL == 32 ? 4 : 1;
+    return NL == 32 ? 4 : (NL == 16 ? 2 : 1);
 }
 // Register cap: 10 warps per SM up to 8 layers, 14 for 16 layers (128 registers: the shared-memory limit is
 // also 14 warps of two subcarriers), none for 32.
@@ -206,7 +225,9 @@ mmse_kernel(const __grid_constant__ MmseArgs g, long long total_sc, const float2
     if (sc0 < total_sc) {                        // else the whole warp is idle until the output rows
         const long long my_sc = sc0 + grp;
         const bool valid = my_sc < total_sc;
-        const long long slot = my_sc / n_sc;
+        long long slot;
+        int my_a;
+        slot_of(my_sc, n_sc, total_sc, slot, my_a);
 
         const float2 *hr = Ht + grp * ht + i * hs;  // own row
         const float2 *hg = Ht + grp * ht;           // the group's rows
@@ -252,7 +273,9 @@ mmse_kernel(const __grid_constant__ MmseArgs g, long long total_sc, const float2
                 const long long sc = sc0 + gg;
                 float2 *dst = Yt + (gg * nd + d) * ys;
                 if (sc < total_sc) {
-                    const long long sl = sc / n_sc, aa = sc - sl * n_sc;
+                    long long sl;
+                    int aa;
+                    slot_of(sc, n_sc, total_sc, sl, aa);
                     const float2 *src = beam + ((sl * g.n_sym + data_symbol(g, g.d_first + d)) * n_sc + aa) * NB;
                     asm volatile(
                         "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
@@ -284,7 +307,9 @@ mmse_kernel(const __grid_constant__ MmseArgs g, long long total_sc, const float2
                 const long long sc = sc0 + gg;
                 float2 *dst = Yt + (gg * nd + d) * ys + (wide ? 2 * c : c);
                 if (sc < total_sc) {
-                    const long long sl = sc / n_sc, aa = sc - sl * n_sc;
+                    long long sl;
+                    int aa;
+                    slot_of(sc, n_sc, total_sc, sl, aa);
                     const float2 *src =
                         beam + ((sl * g.n_sym + data_symbol(g, g.d_first + d)) * n_sc + aa) * nb + (wide ? 2 * c : c);
                     if (wide)
@@ -326,28 +351,33 @@ mmse_kernel(const __grid_constant__ MmseArgs g, long long total_sc, const float2
 
     // ---- 5. x-hat and the Gray decisions, row by row: thread t writes subcarrier cta_sc0 + t % SPC of the rows
     //         (layer l, data symbol d_first + d), l * nd + d = t / SPC, t / SPC + NL, ... (the CTA's WARPS * 32
-    //         threads are NL times its SPC subcarriers), reading x_d[l] from that subcarrier's rows.
-    bool nonfinite = false;
+    //         threads are NL times its SPC subcarriers), reading x_d[l] from that subcarrier's rows. (A layer per
+    //         thread, its symbols in turn, is simpler but writes rows 12 times as far apart: 6 % slower.)
+    float nf = 0.f;   // becomes NaN when a symbol is not finite
     {
         const int s = threadIdx.x % SPC;
         const long long sc = cta_sc0 + s;
         if (sc < total_sc) {
             const int w = s / SPW, gg = s - w * SPW;
             const float2 *yt = reinterpret_cast<const float2 *>(smem_raw + (size_t)w * wsb) + SPW * ht + gg * nd * ys;
-            const long long sl = sc / n_sc, a = sc - sl * n_sc;
-            float2 *xo = xhat + (sl * nl * (long long)g.n_data + g.d_first) * n_sc + a;
-            uint8_t *bo = bits + (sl * nl * (long long)g.n_data + g.d_first) * n_sc + a;
+            long long sl;
+            int a;
+            slot_of(sc, n_sc, total_sc, sl, a);
+            const long long o = (sl * nl * (long long)g.n_data + g.d_first) * n_sc + a;
+            float2 *xo = xhat + o;
+            uint8_t *bo = bits + o;
+            const bool whole = g.n_data == nd;           // the rows of this launch are all rows
             for (int ld = threadIdx.x / SPC; ld < nl * nd; ld += NL) {
                 const int l = ld / nd, d = ld - l * nd;
+                const long long r = (long long)(whole ? ld : l * g.n_data + d) * n_sc;
                 const float2 x = yt[d * ys + l];
-                const long long o = ((long long)l * g.n_data + d) * n_sc;
-                xo[o] = x;
-                bo[o] = det_demap(x, g.qam_bits);
-                if (!isfinite(x.x) || !isfinite(x.y)) nonfinite = true;
+                xo[r] = x;
+                bo[r] = det_demap(x, g.qam_bits);
+                nf = fmaf(x.x, 0.f, fmaf(x.y, 0.f, nf));
             }
         }
     }
-    if (__any_sync(kFull, nonfinite) && lane == 0) atomicOr(&status[0], (unsigned)PUSCH_STATUS_NONFINITE);
+    if (__any_sync(kFull, nf != 0.f) && lane == 0) atomicOr(&status[0], (unsigned)PUSCH_STATUS_NONFINITE);
 }
 
 template <int NL, int ND, int WARPS, int NB>
