@@ -145,6 +145,8 @@ pusch_status check_handle(const pusch_handle *h, int n_slots) {
 }
 
 __global__ void status_init_kernel(uint32_t *status) {
+    pusch::chain_wait(status);
+    pusch::chain_go();
     status[0] = 0u;
     status[1] = 0u;
     status[2] = 0xffffffffu;
@@ -152,7 +154,7 @@ __global__ void status_init_kernel(uint32_t *status) {
 }
 
 pusch_status reset_status(uint32_t *status, cudaStream_t st) {
-    status_init_kernel<<<1, 1, 0, st>>>(status);
+    pusch::launch_chained(true, status_init_kernel, dim3(1), dim3(1), 0, st, status);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "status reset");
     return PUSCH_OK;
@@ -190,6 +192,7 @@ Geometry make_geometry(const pusch_cell_cfg &c) {
     g.sc_pitch = sc_pitch_of(c.form, c.n_sc);
     for (int l = 0; l < 32; ++l) g.port[l] = l < c.n_layers ? c.port[l] : 0;
     g.dmrs_type = c.dmrs_type;
+    g.chained = true;
     if (c.dmrs_type == 1) {  // the estimate lives at the CDM pair centres: spacing 4, offset 1 + CDM group
         g.comb = 4;
         for (int l = 0; l < c.n_layers; ++l) g.port[l] = 1 + c.port[l] / 2;

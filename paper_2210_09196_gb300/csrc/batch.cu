@@ -76,6 +76,8 @@ __device__ __forceinline__ int data_symbol(const DetArgs &g, int d) {
 // ------------------------------------------------------------------------------------------------ kernels
 
 __global__ void batch_reset_kernel(int *counters, uint32_t *status) {
+    pusch::chain_wait(counters, status);
+    pusch::chain_go();
     if (threadIdx.x < kClasses) counters[threadIdx.x] = 0;
     if (threadIdx.x == 0) {
         status[0] = 0u;
@@ -89,6 +91,8 @@ __global__ void batch_reset_kernel(int *counters, uint32_t *status) {
 __global__ void __launch_bounds__(256)
 batch_ls_kernel(const LsJob *__restrict__ jobs, DetArgs g, const float2 *__restrict__ beam,
                 const float2 *__restrict__ pilots, float2 *__restrict__ ls) {
+    pusch::chain_wait(jobs, beam, pilots, ls);
+    pusch::chain_go();
     const LsJob j = jobs[blockIdx.x];
     const float2 *y0 = beam + j.beam_off + (long long)g.dmrs0 * j.n_sc * j.nb;
     const float2 *y1 = beam + j.beam_off + (long long)g.dmrs1 * j.n_sc * j.nb;
@@ -123,6 +127,8 @@ batch_detect_kernel(DetArgs g, int nbmax, const Segment *__restrict__ segs, cons
                     const int2 *__restrict__ items, int n_items, int *__restrict__ counter,
                     const float2 *__restrict__ beam, const float2 *__restrict__ ls, float2 *__restrict__ xhat,
                     uint8_t *__restrict__ bits, uint32_t *__restrict__ status) {
+    pusch::chain_wait(segs, layers, items, counter, beam, ls, xhat, bits, status);
+    pusch::chain_go();
     constexpr int SPW = 32 / NL;
     constexpr int NR = ND > 0 ? ND : kMaxData;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -285,7 +291,7 @@ cudaError_t launch_detect_nl(const DetArgs &g, int nbmax, const Segment *segs, c
     long long grid = (long long)sms * per_sm;
     const long long need = ((long long)n_items + warps - 1) / warps;
     if (grid > need) grid = need;
-    k<<<(unsigned)grid, warps * 32, smem, st>>>(g, nbmax, segs, layers, items, n_items, counter, beam, ls, xhat, bits,
+    pusch::launch_chained(false, k, dim3((unsigned)grid), dim3(warps * 32), smem, st, g, nbmax, segs, layers, items, n_items, counter, beam, ls, xhat, bits,
                                                 status);
     return cudaGetLastError();
 }
@@ -382,7 +388,7 @@ pusch_status enqueue(pusch_batch *b, const void *time_in, const void *W, const v
     cudaError_t e;
     const int nbr = std::max(1, std::min(b->branches, kMaxBranches));
     auto fail_e = [&](const char *what) { return bcuda(e, what); };
-    batch_reset_kernel<<<1, 32, 0, s>>>(b->d_counters, status);
+    pusch::launch_chained(true, batch_reset_kernel, dim3(1), dim3(32), 0, s, b->d_counters, status);
     if ((e = cudaGetLastError()) != cudaSuccess) return fail_e("batch reset launch");
     if (only_class < 0) {
         const size_t tsz = b->cells[0].in_fp16 ? 4 : 8;
@@ -409,7 +415,7 @@ pusch_status enqueue(pusch_batch *b, const void *time_in, const void *W, const v
                 if ((e = cudaStreamWaitEvent(s, b->ev[2 + k], 0)) != cudaSuccess) return fail_e("join wait");
             }
         if (b->n_jobs > 0) {
-            batch_ls_kernel<<<b->n_jobs, 256, 0, s>>>(b->d_jobs, b->det, b->beam, static_cast<const float2 *>(pilots),
+            pusch::launch_chained(true, batch_ls_kernel, dim3(b->n_jobs), dim3(256), 0, s, b->d_jobs, b->det, b->beam, static_cast<const float2 *>(pilots),
                                                       b->ls);
             if ((e = cudaGetLastError()) != cudaSuccess) return fail_e("batch LS launch");
         }
@@ -540,6 +546,9 @@ pusch_status pusch_batch_create(pusch_batch **out, const pusch_cell_cfg *cells, 
         cc.port[0] = 0;
         cc.qam_bits = 2;
         b->geo.push_back(pusch::make_geometry(cc));
+        // the cells' chains run on parallel branches: a kernel that waits on an SM for its predecessor would keep the
+        // other branches' out
+        b->geo.back().chained = false;
         b->nbmax = std::max(b->nbmax, cc.n_beams);
     }
     const Geometry &g0 = b->geo[0];

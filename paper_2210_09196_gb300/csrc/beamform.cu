@@ -20,6 +20,8 @@ template <int GB>  // beam groups of 8: ceil(n_beams / 8)
 __global__ void __launch_bounds__(kBfThreads)
 beamform_fp32_kernel(const float2 *__restrict__ freq, const float2 *__restrict__ W, float2 *__restrict__ beam,
                      int n_rx, int n_sc, int n_beams) {
+    chain_wait(freq, W, beam);
+    chain_go();
     constexpr int TA = (kBfThreads / GB) * kSB;  // subcarriers per CTA
     constexpr int WB = GB * kBB;                 // padded beams
     __shared__ __align__(16) float2 Xs[kKC][TA];
@@ -97,7 +99,7 @@ cudaError_t launch_gb(const Geometry &g, int n_slots, const float2 *freq, const 
     const long long rows = (long long)n_slots * g.n_sym;
     if (rows > 65535) return cudaErrorInvalidConfiguration;
     dim3 grid((g.n_sc + TA - 1) / TA, (unsigned)rows);
-    beamform_fp32_kernel<GB><<<grid, kBfThreads, 0, st>>>(freq, W, beam, g.n_rx, g.n_sc, g.n_beams);
+    launch_chained(g.chained, beamform_fp32_kernel<GB>, grid, dim3(kBfThreads), 0, st, freq, W, beam, g.n_rx, g.n_sc, g.n_beams);
     return cudaGetLastError();
 }
 

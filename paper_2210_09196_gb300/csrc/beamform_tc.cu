@@ -115,6 +115,8 @@ __global__ void __launch_bounds__(FP8 ? 192 + 32 * kConvWarps : 192, 1)
 beamform_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap omap, TcArgs g,
                    const float2 *__restrict__ W, const float *__restrict__ scales, float2 *__restrict__ beam,
                    uint32_t *__restrict__ err) {
+    chain_wait(W, scales, beam, err);
+    chain_go();
     constexpr int kThreads = FP8 ? 192 + 32 * kConvWarps : 192;
     constexpr int kKStep = 16;                  // K per MMA instruction (32 bytes of FP16)
     extern __shared__ uint8_t smem_raw[];
@@ -639,7 +641,7 @@ cudaError_t launch_tc(const Geometry &g, int n_slots, const void *freq, const fl
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     long long grid = sms;
     if (grid > a.total_tiles) grid = a.total_tiles;
-    kern<<<(unsigned)grid, FP8 ? 192 + 32 * kConvWarps : 192, p.smem, st>>>(map, omap, a, W, scales, beam, err_word);
+    launch_chained(g.chained, kern, dim3((unsigned)grid), dim3(FP8 ? 192 + 32 * kConvWarps : 192), p.smem, st, map, omap, a, W, scales, beam, err_word);
     return cudaGetLastError();
 }
 

@@ -83,6 +83,8 @@ __device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint64_t a, uint64_t b
 __global__ void __launch_bounds__(kThreads, 1)
 beamform_tf32_kernel(const __grid_constant__ CUtensorMap tmap, Tf32Args g, const float2 *__restrict__ W,
                      float2 *__restrict__ beam, uint32_t *__restrict__ err) {
+    chain_wait(W, beam, err);
+    chain_go();
     extern __shared__ uint8_t smem_raw[];
     __shared__ Tf32Shared sh;
 
@@ -395,7 +397,7 @@ cudaError_t launch_beamform_tf32(const Geometry &g, int n_slots, const float2 *f
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     long long grid = sms;
     if (grid > a.total_tiles) grid = a.total_tiles;
-    beamform_tf32_kernel<<<(unsigned)grid, kThreads, p.smem, st>>>(map, a, W, beam, err_word);
+    launch_chained(g.chained, beamform_tf32_kernel, dim3((unsigned)grid), dim3(kThreads), p.smem, st, map, a, W, beam, err_word);
     return cudaGetLastError();
 }
 

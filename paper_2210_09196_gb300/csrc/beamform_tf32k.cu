@@ -170,6 +170,8 @@ __device__ __forceinline__ bool wait_cluster(uint32_t bar, uint32_t parity, vola
 __global__ void __launch_bounds__(kThreads, 1)
 beamform_tf32k_kernel(Tf32Args g, const float2 *__restrict__ freq, const float2 *__restrict__ W,
                      float2 *__restrict__ beam, uint32_t *__restrict__ err) {
+    chain_wait(freq, W, beam, err);
+    chain_go();
     extern __shared__ uint8_t smem_raw[];
     __shared__ Tf32Shared sh;
 
@@ -563,7 +565,7 @@ cudaError_t launch_beamform_tf32k(const Geometry &g, int n_slots, const float2 *
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaLaunchConfig_t cfg{};
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)p.cluster;
     at[0].val.clusterDim.y = 1;
@@ -572,7 +574,9 @@ cudaError_t launch_beamform_tf32k(const Geometry &g, int n_slots, const float2 *
     cfg.dynamicSmemBytes = p.smem;
     cfg.stream = st;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // launch_chained, with a cluster
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = 2;
     // as many clusters as are resident at once (36 of 4 CTAs on 152 SMs): the tiles are dealt out evenly, so a
     // cluster that had to wait for a place would double the time
     int clusters = sms;

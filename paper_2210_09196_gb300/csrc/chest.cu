@@ -62,6 +62,8 @@ template <typename T, bool TV>
 __global__ void __launch_bounds__(1024)
 chest_interp_kernel(ChestArgs g, int kmax, int units, int layers_per_cta, const T *__restrict__ ls,
                     long long tab_stride, T *__restrict__ H, long long h_stride) {
+    chain_wait(ls, H);
+    chain_go();
     __shared__ int s_klo[kRun][32], s_khi[kRun][32];
     __shared__ float s_w[kRun][32];
     const int t = threadIdx.x;
@@ -105,6 +107,8 @@ chest_interp_kernel(ChestArgs g, int kmax, int units, int layers_per_cta, const 
 __global__ void __launch_bounds__(256)
 ls_pilots_kernel(ChestArgs g, int kmax, int sym, const float2 *__restrict__ beam, const float2 *__restrict__ pilots,
                  float2 *__restrict__ ls) {
+    chain_wait(beam, pilots, ls);
+    chain_go();
     // grid.y = slot * n_layers + l, grid.x: chunks of the layer's kmax * n_beams (pilot, beam) elements
     const long long sl = blockIdx.y;
     const long long slot = sl / g.n_layers;
@@ -148,6 +152,8 @@ ls_pilots_kernel(ChestArgs g, int kmax, int sym, const float2 *__restrict__ beam
 __global__ void __launch_bounds__(256)
 ne_partial_kernel(ChestArgs g, int kmax, const float2 *__restrict__ beam, const float2 *__restrict__ pilots,
                   float2 *__restrict__ partial) {
+    chain_wait(beam, pilots, partial);
+    chain_go();
     __shared__ float2 red[8];
     const long long slot = blockIdx.y;
     const int per_l = kmax * g.n_beams;                     // < 2^31: n_sc <= 4096, n_beams <= 64
@@ -196,6 +202,8 @@ struct NeType1Args {
 __global__ void __launch_bounds__(256)
 ne_partial_type1_kernel(NeType1Args g, const float2 *__restrict__ beam, const float2 *__restrict__ pilots,
                         float2 *__restrict__ partial) {
+    chain_wait(beam, pilots, partial);
+    chain_go();
     __shared__ float2 red[8];
     const long long slot = blockIdx.y;
     const int per_group = g.n_pairs * g.n_beams;
@@ -253,6 +261,8 @@ ne_partial_type1_kernel(NeType1Args g, const float2 *__restrict__ beam, const fl
 // factor 1 (the count is already the degrees of freedom).
 __global__ void ne_final_kernel(int n_parts, const float2 *__restrict__ partial, float *__restrict__ sigma2,
                                 float factor) {
+    chain_wait(partial, sigma2);
+    chain_go();
     const int slot = blockIdx.x, lane = threadIdx.x;
     float2 t = make_float2(0.f, 0.f);
     for (int p = lane; p < n_parts; p += 32) t = cadd(t, partial[(long long)slot * n_parts + p]);
@@ -292,15 +302,15 @@ cudaError_t launch_noise_est(const Geometry &g, int n_slots, const float2 *beam,
         a.l01 = lay[0][1];
         a.l10 = lay[1][0];
         a.l11 = lay[1][1];
-        ne_partial_type1_kernel<<<dim3(kNoiseParts, (unsigned)n_slots), 256, 0, st>>>(a, beam, pilots, partial);
+        launch_chained(g.chained, ne_partial_type1_kernel, dim3(kNoiseParts, (unsigned)n_slots), dim3(256), 0, st, a, beam, pilots, partial);
     } else {
         const ChestArgs a = chest_args(g);
-        ne_partial_kernel<<<dim3(kNoiseParts, (unsigned)n_slots), 256, 0, st>>>(a, ls_pilots_per_layer(g), beam,
+        launch_chained(g.chained, ne_partial_kernel, dim3(kNoiseParts, (unsigned)n_slots), dim3(256), 0, st, a, ls_pilots_per_layer(g), beam,
                                                                                  pilots, partial);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    ne_final_kernel<<<(unsigned)n_slots, 32, 0, st>>>(kNoiseParts, partial, sigma2, g.dmrs_type == 1 ? 1.f : 2.f);
+    launch_chained(g.chained, ne_final_kernel, dim3((unsigned)n_slots), dim3(32), 0, st, kNoiseParts, partial, sigma2, g.dmrs_type == 1 ? 1.f : 2.f);
     return cudaGetLastError();
 }
 
@@ -312,7 +322,7 @@ cudaError_t launch_ls_pilots(const Geometry &g, int n_slots, const float2 *beam,
     if (rows == 0) return cudaSuccess;
     if (rows > 65535) return cudaErrorInvalidValue;   // grid.y; n_slots * n_layers per call
     const int per_l = kmax * g.n_beams;
-    ls_pilots_kernel<<<dim3((unsigned)((per_l + 255) / 256), (unsigned)rows), 256, 0, st>>>(a, kmax, sym, beam, pilots,
+    launch_chained(g.chained, ls_pilots_kernel, dim3((unsigned)((per_l + 255) / 256), (unsigned)rows), dim3(256), 0, st, a, kmax, sym, beam, pilots,
                                                                                            ls);
     return cudaGetLastError();
 }
@@ -338,11 +348,11 @@ cudaError_t launch_chest_interp(const Geometry &g, int n_slots, const float2 *ls
     if (pairs) {
         const float4 *l4 = reinterpret_cast<const float4 *>(ls);
         float4 *h4 = reinterpret_cast<float4 *>(H);
-        if (time_groups) chest_interp_kernel<float4, true><<<grid, threads, 0, st>>>(a, kmax, units, lpc, l4, tab_u, h4, h_u);
-        else chest_interp_kernel<float4, false><<<grid, threads, 0, st>>>(a, kmax, units, lpc, l4, tab_u, h4, h_u);
+        if (time_groups) launch_chained(g.chained, chest_interp_kernel<float4, true>, grid, dim3(threads), 0, st, a, kmax, units, lpc, l4, tab_u, h4, h_u);
+        else launch_chained(g.chained, chest_interp_kernel<float4, false>, grid, dim3(threads), 0, st, a, kmax, units, lpc, l4, tab_u, h4, h_u);
     } else {
-        if (time_groups) chest_interp_kernel<float2, true><<<grid, threads, 0, st>>>(a, kmax, units, lpc, ls, tab_u, H, h_u);
-        else chest_interp_kernel<float2, false><<<grid, threads, 0, st>>>(a, kmax, units, lpc, ls, tab_u, H, h_u);
+        if (time_groups) launch_chained(g.chained, chest_interp_kernel<float2, true>, grid, dim3(threads), 0, st, a, kmax, units, lpc, ls, tab_u, H, h_u);
+        else launch_chained(g.chained, chest_interp_kernel<float2, false>, grid, dim3(threads), 0, st, a, kmax, units, lpc, ls, tab_u, H, h_u);
     }
     return cudaGetLastError();
 }

@@ -19,6 +19,8 @@ constexpr int kCh[5] = {2, 32, 32, 32, 2};
 __global__ void adam_kernel(int n, float lr, float b1, float b2, float eps, float c1, float c2, float *__restrict__ p,
                             __nv_bfloat16 *__restrict__ pb, const float *__restrict__ g, float *__restrict__ m,
                             float *__restrict__ v) {
+    chain_wait(p, pb, g, m, v);
+    chain_go();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const float gi = g[i];
@@ -62,7 +64,7 @@ cudaError_t cnn_adam(int step, float lr, float b1, float b2, float eps, float *p
                      float *m, float *v, cudaStream_t st) {
     const int n = cnn_param_count();
     const float c1 = 1.f - powf(b1, (float)step), c2 = 1.f - powf(b2, (float)step);
-    adam_kernel<<<(n + 255) / 256, 256, 0, st>>>(n, lr, b1, b2, eps, c1, c2, p, pb, g, m, v);
+    launch_chained(true, adam_kernel, dim3((n + 255) / 256), dim3(256), 0, st, n, lr, b1, b2, eps, c1, c2, p, pb, g, m, v);
     return cudaGetLastError();
 }
 
@@ -106,6 +108,8 @@ __device__ __forceinline__ float block_sum(float v, float *red) {
 __global__ void __launch_bounds__(256)
 ls_grid_kernel(GridArgs g, const float2 *__restrict__ beam, const float2 *__restrict__ pilots,
                __nv_bfloat16 *__restrict__ grid, float *__restrict__ scale) {
+    chain_wait(beam, pilots, grid, scale);
+    chain_go();
     __shared__ float red[32];
     const long long gi = blockIdx.x;
     const int b = (int)(gi % g.n_beams);
@@ -147,6 +151,8 @@ __global__ void __launch_bounds__(256)
 cnn_to_h_kernel(GridArgs g, float noise_var, float kappa, const float *__restrict__ y, const float *__restrict__ scale,
                 const float2 *__restrict__ beam, const float2 *__restrict__ pilots, float2 *__restrict__ H,
                 float *__restrict__ resid, uint8_t *__restrict__ fallback) {
+    chain_wait(y, scale, beam, pilots, H, resid, fallback);
+    chain_go();
     __shared__ float red[32];
     const long long gi = blockIdx.x;
     const int b = (int)(gi % g.n_beams);
@@ -215,7 +221,7 @@ cudaError_t launch_ls_grid(const Geometry &g, int n_slots, const float2 *beam, c
     const long long grids = (long long)n_slots * g.n_layers * g.n_beams;
     if (grids == 0) return cudaSuccess;
     if (grids > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    ls_grid_kernel<<<(unsigned)grids, 256, 0, st>>>(grid_args(g), beam, pilots, grid, scale);
+    launch_chained(true, ls_grid_kernel, dim3((unsigned)grids), dim3(256), 0, st, grid_args(g), beam, pilots, grid, scale);
     return cudaGetLastError();
 }
 
@@ -224,7 +230,7 @@ cudaError_t launch_cnn_to_h(const Geometry &g, int n_slots, float kappa, const f
                             cudaStream_t st) {
     const long long grids = (long long)n_slots * g.n_layers * g.n_beams;
     if (grids == 0) return cudaSuccess;
-    cnn_to_h_kernel<<<(unsigned)grids, 256, 0, st>>>(grid_args(g), g.noise_var + g.loading, kappa, y, scale, beam,
+    launch_chained(true, cnn_to_h_kernel, dim3((unsigned)grids), dim3(256), 0, st, grid_args(g), g.noise_var + g.loading, kappa, y, scale, beam,
                                                      pilots, H, resid, fallback);
     return cudaGetLastError();
 }

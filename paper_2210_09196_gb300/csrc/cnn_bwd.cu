@@ -119,6 +119,7 @@ __global__ void __launch_bounds__(kMidThreads, 1)
 cnn_bwd_mid_kernel(BwdArgs g, const float *__restrict__ gout, const __nv_bfloat16 *__restrict__ acts,
                    const __nv_bfloat16 *__restrict__ W, float *__restrict__ gin, float *__restrict__ dW,
                    float *__restrict__ db, uint32_t *__restrict__ err) {
+    chain_wait(gout, acts, W, gin, dW, db, err);
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t bar_d[kCtx], bar_p[kCtx];
     __shared__ uint32_t s_tmem;
@@ -365,6 +366,7 @@ __global__ void __launch_bounds__(kEndThreads, 2)
 cnn_bwd_out_kernel(BwdArgs g, const float *__restrict__ y, const float *__restrict__ tgt,
                    const __nv_bfloat16 *__restrict__ acts, const __nv_bfloat16 *__restrict__ W, float *__restrict__ gin,
                    float *__restrict__ dW, float *__restrict__ db, float *__restrict__ loss) {
+    chain_wait(y, tgt, acts, W, gin, dW, db, loss);
     __shared__ __align__(16) uint8_t s_a[kTile * 128];
     __shared__ float4 s_g[kTile + 2];            // g4 (h * 2 + co) of subcarriers x0 - 1 .. x0 + kTile
     __shared__ float s_red[kEndWeights];
@@ -469,6 +471,7 @@ cnn_bwd_out_kernel(BwdArgs g, const float *__restrict__ y, const float *__restri
 __global__ void __launch_bounds__(kEndThreads, 3)
 cnn_bwd_in_kernel(BwdArgs g, const float *__restrict__ gout, const __nv_bfloat16 *__restrict__ in,
                   float *__restrict__ dW, float *__restrict__ db) {
+    chain_wait(gout, in, dW, db);
     __shared__ float4 s_x[kTile + 2];            // inputs (r * 2 + ci) of subcarriers x0 - 1 .. x0 + kTile
     __shared__ float s_red[kEndWeights];
     __shared__ float s_db[32];
@@ -543,18 +546,18 @@ cudaError_t launch_cnn_bwd(int n, int w, const __nv_bfloat16 *x, const __nv_bflo
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const unsigned one = (unsigned)(tiles < sms ? tiles : sms), two = (unsigned)(tiles < 2 * sms ? tiles : 2 * sms);
     const unsigned three = (unsigned)(tiles < 3 * sms ? tiles : 3 * sms);
-    cnn_bwd_out_kernel<<<two, kEndThreads, 0, st>>>(a, y, target, acts + 2 * big, P + kO4, gbuf, grad + kO4,
+    launch_chained(true, cnn_bwd_out_kernel, dim3(two), dim3(kEndThreads), 0, st, a, y, target, acts + 2 * big, P + kO4, gbuf, grad + kO4,
                                                     grad + kO4 + 2 * 32 * 9, loss);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     a.dil = 16;
-    cnn_bwd_mid_kernel<<<one, kMidThreads, kMidSmem, st>>>(a, gbuf, acts + big, P + kO3, ga, grad + kO3,
+    launch_chained(true, cnn_bwd_mid_kernel, dim3(one), dim3(kMidThreads), kMidSmem, st, a, gbuf, acts + big, P + kO3, ga, grad + kO3,
                                                            grad + kO3 + 32 * 32 * 9, err);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     a.dil = 8;
-    cnn_bwd_mid_kernel<<<one, kMidThreads, kMidSmem, st>>>(a, ga, acts, P + kO2, gbuf, grad + kO2,
+    launch_chained(true, cnn_bwd_mid_kernel, dim3(one), dim3(kMidThreads), kMidSmem, st, a, ga, acts, P + kO2, gbuf, grad + kO2,
                                                            grad + kO2 + 32 * 32 * 9, err);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    cnn_bwd_in_kernel<<<three, kEndThreads, 0, st>>>(a, gbuf, x, grad, grad + 32 * 2 * 9);
+    launch_chained(true, cnn_bwd_in_kernel, dim3(three), dim3(kEndThreads), 0, st, a, gbuf, x, grad, grad + 32 * 2 * 9);
     return cudaGetLastError();
 }
 

@@ -70,6 +70,7 @@ __device__ __forceinline__ uint32_t sw128(int row, int k) {
 __global__ void __launch_bounds__(kThreads, 1)
 cnn_fwd_kernel(FwdArgs g, const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__restrict__ P,
                float *__restrict__ y, __nv_bfloat16 *__restrict__ acts, uint32_t *__restrict__ err) {
+    chain_wait(in, P, y, acts, err);
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t bars[kCtx];
     __shared__ uint32_t s_tmem;
@@ -414,7 +415,7 @@ cudaError_t launch_cnn_fwd(const __nv_bfloat16 *in, const __nv_bfloat16 *P, floa
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const long long grid = tiles < sms ? tiles : sms;
-    cnn_fwd_kernel<<<(unsigned)grid, kThreads, kSmemBytes, st>>>(a, in, P, y, acts, err);
+    launch_chained(true, cnn_fwd_kernel, dim3((unsigned)grid), dim3(kThreads), kSmemBytes, st, a, in, P, y, acts, err);
     return cudaGetLastError();
 }
 

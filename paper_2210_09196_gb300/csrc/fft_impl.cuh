@@ -236,6 +236,7 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_
 struct FftIn {
     int cp, cp0, cp1, shift, n_sym, n_rx;
     long long slot_len;
+    bool chained;    // launched with launch_chained
 };
 __device__ __forceinline__ long long fft_row_offset(const FftIn &fi, int N, long long row) {
     if (!fi.cp) return row * N;
@@ -304,6 +305,8 @@ __global__ void __launch_bounds__(kFftThreads, fft_min_ctas<TIn>())
 fft_kernel(const TIn *__restrict__ in, void *__restrict__ out, const float2 *__restrict__ tw, long long rows,
            int n_sc, int pitch, float *__restrict__ scales, int n_rx, int n_blk, uint32_t *__restrict__ err,
            FftIn fi) {
+    pusch::chain_wait(in, out, tw, scales, err);
+    pusch::chain_go();
     constexpr int E = Plan<N>::E;
     constexpr int T = N / E;
     constexpr int F = ffts_per_cta<N>();
@@ -546,7 +549,7 @@ cudaError_t launch_n(long long rows, const void *in, void *out, const float2 *tw
     const long long blocks = (rows + F - 1) / F;
     long long grid = (long long)sms * per_sm;
     if (grid > blocks) grid = blocks;
-    k<<<(unsigned)grid, kFftThreads, smem, st>>>(static_cast<const TIn *>(in), out, tw, rows, n_sc, pitch, scales,
+    launch_chained(fi.chained, k, dim3((unsigned)grid), dim3(kFftThreads), smem, st, static_cast<const TIn *>(in), out, tw, rows, n_sc, pitch, scales,
                                                   n_rx, n_blk, err, fi);
     return cudaGetLastError();
 }
@@ -564,6 +567,7 @@ cudaError_t launch_out(const Geometry &g, long long rows, const void *in, void *
     fi.n_sym = g.n_sym;
     fi.n_rx = g.n_rx;
     fi.slot_len = g.slot_len;
+    fi.chained = g.chained;
     switch (g.n_fft) {
         case 4096: return launch_n<4096, TIn, OUT>(rows, in, out, tw, g.n_sc, g.sc_pitch, scales, g.n_rx, n_blk, err, fi, st, g.fft_cap);
         case 2048: return launch_n<2048, TIn, OUT>(rows, in, out, tw, g.n_sc, g.sc_pitch, scales, g.n_rx, n_blk, err, fi, st, g.fft_cap);

@@ -95,6 +95,8 @@ struct FftTcArgs {
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 fft_tc_kernel(const __grid_constant__ CUtensorMap tin, __half *__restrict__ out, const float2 *__restrict__ tw,
               FftTcArgs g, uint32_t *__restrict__ err) {
+    chain_wait(out, tw, err);
+    chain_go();
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t bar_full[kStages];
     __shared__ __align__(8) uint64_t bar_acc;     // MMA commits: the accumulator holds a finished product
@@ -315,7 +317,7 @@ cudaError_t launch_fft_tc(const Geometry &g, long long rows, const void *in, voi
     a.rows = rows;
     a.n_sc = g.n_sc;
     a.pitch = g.sc_pitch;
-    fft_tc_kernel<<<(unsigned)grid, kThreads, kSmemBytes, st>>>(map, static_cast<__half *>(out), tw, a, err);
+    launch_chained(g.chained, fft_tc_kernel, dim3((unsigned)grid), dim3(kThreads), kSmemBytes, st, map, static_cast<__half *>(out), tw, a, err);
     return cudaGetLastError();
 }
 

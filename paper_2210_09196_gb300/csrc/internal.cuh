@@ -41,6 +41,43 @@ __device__ __forceinline__ void cfms(float2 &acc, float2 a, float2 b) {
     acc.y = fmaf(-a.x, b.y, fmaf(-a.y, b.x, acc.y));
 }
 
+// ------------------------------------------------------------------------------------- chained launches
+// Programmatic dependent launch: a kernel launched with launch_chained may start while the kernel before it on the
+// stream is still running, and waits for it inside (chain_wait, which every such kernel executes before it touches
+// global memory), so that launch latency, block scheduling and what a kernel sets up before the wait overlap the tail
+// of the kernel before. chain_wait then lets the next kernel in line start the same way; nothing before a kernel's own
+// wait has therefore seen the end of anything but the kernels before its predecessor. The pointers a kernel works
+// through are given to chain_wait, which redefines them behind the wait, so that no load through them, read-only or
+// not, can be moved before it. Measured (GB300), against ordinary launches: one slot of the small cell (7 kernels) 38 ->
+// 26 us, estimation and detection of 2 massive slots (5 kernels) 202 -> 186 us, 16 deployment slots 421 -> 412 us.
+template <typename T>
+__device__ __forceinline__ void redefine_pointer(T &p) {
+    asm volatile("" : "+l"(p) : : "memory");
+}
+template <typename... T>
+__device__ __forceinline__ void chain_wait(T &...p) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    (redefine_pointer(p), ...);
+}
+// Lets the next kernel of the chain start (all CTAs have to have called it or ended).
+__device__ __forceinline__ void chain_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// chained = false: an ordinary launch (the waits inside pass at once).
+template <typename... P, typename... A>
+inline cudaError_t launch_chained(bool chained, void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                  A... args) {
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = chained ? 1 : 0;
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
+}
+
 // ---------------------------------------------------------------------------------- derived geometry
 struct Geometry {
     int n_rx, n_fft, n_sc, n_beams, n_layers, comb, qam_bits, in_fp16, form, n_sym;
@@ -60,6 +97,7 @@ struct Geometry {
     int dmrs_type;                // 1: 3GPP type-1 DMRS; comb / port then give the CDM pair centres (4, 1 + group)
     // launch shapes (pusch_autotune; 0 = the built-in choice)
     int fft_cap;                  // FFT CTAs per SM at most
+    bool chained;                 // kernels may start before their predecessor ends (launch_chained)
     int det_warps;                // warps per CTA of the 12-data-symbol detector (0 = the class default)
 };
 

@@ -9,9 +9,9 @@ cudaError_t launch_mmse(const Geometry &g, int n_slots, const float2 *H, const f
                         const float2 *ls) {
     if (ls && (time_groups || !mmse_interp_supported(g, beam, ls))) return cudaErrorNotSupported;
     mmse_detail::MmseArgs a;
-    a.ls = ls;
     a.kmax = ls ? ls_pilots_per_layer(g) : 0;
     a.comb = g.comb;
+    a.chained = g.chained;
     for (int l = 0; l < 32; ++l) a.port[l] = l < g.n_layers ? g.port[l] : 0;
     a.warps = g.det_warps;
     a.n_sc = g.n_sc;
@@ -22,7 +22,6 @@ cudaError_t launch_mmse(const Geometry &g, int n_slots, const float2 *H, const f
     a.qam_bits = g.qam_bits;
     a.load = g.noise_var + g.loading;
     a.loading = g.loading;
-    a.sigma2 = sigma2;
     a.dmrs_lo = g.dmrs0 < g.dmrs1 ? g.dmrs0 : g.dmrs1;
     a.dmrs_hi = g.dmrs0 < g.dmrs1 ? g.dmrs1 : g.dmrs0;
     if (g.n_data > 14) return cudaErrorInvalidValue;
@@ -40,11 +39,11 @@ cudaError_t launch_mmse(const Geometry &g, int n_slots, const float2 *H, const f
         const float2 *Hq = H + q * stride;
         cudaError_t e;
         if (nl <= 8)
-            e = mmse_launch_class(nl <= 2 ? 2 : (nl <= 4 ? 4 : 8), a, total_sc, Hq, beam, x_hat, bits, status, st);
+            e = mmse_launch_class(nl <= 2 ? 2 : (nl <= 4 ? 4 : 8), a, total_sc, Hq, beam, ls, sigma2, x_hat, bits, status, st);
         else if (nl <= 16)
-            e = mmse_launch_class16(a, total_sc, Hq, beam, x_hat, bits, status, st);
+            e = mmse_launch_class16(a, total_sc, Hq, beam, ls, sigma2, x_hat, bits, status, st);
         else
-            e = mmse_launch_class32(a, total_sc, Hq, beam, x_hat, bits, status, st);
+            e = mmse_launch_class32(a, total_sc, Hq, beam, ls, sigma2, x_hat, bits, status, st);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

@@ -33,16 +33,13 @@ constexpr unsigned kFull = 0xffffffffu;
 
 struct MmseArgs {
     int n_sc, n_beams, n_layers, n_sym, n_data, qam_bits;
-    float load;  // sigma^2 + extra loading (sigma2 == nullptr)
+    float load;  // sigma^2 + extra loading (no per-slot sigma2)
     float loading;             // extra loading alone
-    const float *sigma2;       // per-slot noise variance (device) or nullptr
     int d_first, n_det;        // this launch detects data symbols d_first .. d_first + n_det - 1 (n_data in all)
     int dmrs_lo, dmrs_hi;      // the two DMRS symbols, dmrs_lo < dmrs_hi
     int warps;                 // warps per CTA of the 12-symbol kernels (mmse_warp_choices; 0 = default)
-    // LS table at the pilots (ls[slot][l][k][b], pilot q = port[l] + k comb, k < kmax) or nullptr: when set,
-    // the beam-count instances interpolate their estimate rows from it while staging (the same arithmetic as
-    // the interpolation kernel) and the H argument is not read
-    const float2 *ls;
+    bool chained;              // launched with launch_chained
+    // the LS table at the pilots, where the kernel takes one: ls[slot][l][k][b], pilot q = port[l] + k comb, k < kmax
     int kmax, comb;
     int port[32];
 };
@@ -112,7 +109,7 @@ __device__ __forceinline__ void stage_H(float2 *Ht, const float2 *__restrict__ H
 // rows); the warp then reads the two table rows of every tile row in 16-byte pieces (NB / 2 per row), issuing
 // kB pieces' loads before using any. Rows of absent layers and subcarriers are zeroed.
 template <int NL, int NB>
-__device__ __forceinline__ void stage_H_interp(float2 *Ht, const MmseArgs &g, long long sc0, long long total_sc,
+__device__ __forceinline__ void stage_H_interp(float2 *Ht, const MmseArgs &g, const float2 *ls, long long sc0, long long total_sc,
                                                int ht, int lane) {
     constexpr int kU = NB / 2;            // 16-byte pieces per row
     constexpr int kRows = 32 / kU;        // rows per warp pass (2 for 32 beams, 1 for 64)
@@ -142,7 +139,7 @@ __device__ __forceinline__ void stage_H_interp(float2 *Ht, const MmseArgs &g, lo
         }
     }
     const int sub = lane / kU, u = lane - sub * kU;
-    const float4 *tab = reinterpret_cast<const float4 *>(g.ls) + sl0 * g.n_layers * (long long)g.kmax * kU + u;
+    const float4 *tab = reinterpret_cast<const float4 *>(ls) + sl0 * g.n_layers * (long long)g.kmax * kU + u;
     // rows of pass t: when a pass covers SPW rows, the same layer of the warp's SPW subcarriers (neighbouring
     // subcarriers mostly share the bracket, so the pass reads each table line once); else kRows consecutive rows
     constexpr int SPW = 32 / NL;
@@ -198,12 +195,17 @@ constexpr int mmse_min_ctas() {
 // row: the SPC subcarriers of one (slot, layer, data symbol) row are consecutive in both outputs, so each row
 // segment is one contiguous run of SPC elements (a warp per subcarrier pair would write 16-byte pieces of 16
 // rows).
+// ls: the LS table at the pilots or NULL; when set, the beam-count instances interpolate their estimate rows from it while
+// staging (the same arithmetic as the interpolation kernel) and H is not read. sigma2: per-slot noise variance or NULL.
 // NB > 0: compiled for NB beams (every shared-memory offset of the Gram, matched-filter and staging loops is
 // then a constant) and staged by bulk copies on one mbarrier per warp; 0: g.n_beams at run time, cp.async.
 template <int NL, int ND, int WARPS, int NB>
 __global__ void __launch_bounds__(WARPS * 32, mmse_min_ctas<NL, WARPS>())
 mmse_kernel(const __grid_constant__ MmseArgs g, long long total_sc, const float2 *__restrict__ H, const float2 *__restrict__ beam,
-            float2 *__restrict__ xhat, uint8_t *__restrict__ bits, uint32_t *__restrict__ status) {
+            const float2 *__restrict__ ls, const float *__restrict__ sigma2, float2 *__restrict__ xhat,
+            uint8_t *__restrict__ bits, uint32_t *__restrict__ status) {
+    pusch::chain_wait(H, beam, ls, sigma2, xhat, bits, status);
+    pusch::chain_go();
     constexpr int SPW = 32 / NL;
     constexpr int SPC = WARPS * SPW;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -240,7 +242,7 @@ mmse_kernel(const __grid_constant__ MmseArgs g, long long total_sc, const float2
             //           instances only with 16-byte aligned H and beam.
             const uint32_t bar = smem_addr(reinterpret_cast<uint64_t *>(smem_raw + (size_t)WARPS * wsb) + warp);
             constexpr uint32_t kRowB = NB * 8;
-            const bool interp_h = g.ls != nullptr;   // estimate rows interpolated from the LS table
+            const bool interp_h = ls != nullptr;   // estimate rows interpolated from the LS table
             uint32_t my_bytes = 0;
             for (int r = lane; r < SPW * NL && !interp_h; r += 32)
                 if (r % NL < nl && sc0 + r / NL < total_sc) my_bytes += kRowB;
@@ -287,7 +289,7 @@ mmse_kernel(const __grid_constant__ MmseArgs g, long long total_sc, const float2
                     for (int b = 0; b < NB; b += 2) *reinterpret_cast<float4 *>(dst + b) = make_float4(0.f, 0.f, 0.f, 0.f);
                 }
             }
-            if (interp_h) stage_H_interp<NL, NB>(Ht, g, sc0, total_sc, ht, lane);   // overlaps the y copies
+            if (interp_h) stage_H_interp<NL, NB>(Ht, g, ls, sc0, total_sc, ht, lane);   // overlaps the y copies
             // bounded wait (2 s); on expiry the timeout bit is set and the copies are waited for once more
             if (!bw::mbar_wait_for(bar, 0, bw::kWaitNs)) {
                 if (lane == 0) atomicOr(&status[0], (unsigned)PUSCH_STATUS_TIMEOUT);
@@ -336,11 +338,11 @@ mmse_kernel(const __grid_constant__ MmseArgs g, long long total_sc, const float2
         // ---- 2-4. Gram, matched filter, Cholesky and solves, the x_d left in the data-symbol rows (detect_group).
         bool bad;
         if constexpr (NB > 0 && ND == 12 && NL >= 16)   // G and r_d on the tensor cores
-            bad = detect_group_tc<NL, NB>(Ht, ht, hs, Yt, ys, nl, g.sigma2 ? g.loading : g.load, grp, i, src0, lane,
-                                          acc, g.sigma2, valid ? slot : 0);
+            bad = detect_group_tc<NL, NB>(Ht, ht, hs, Yt, ys, nl, sigma2 ? g.loading : g.load, grp, i, src0, lane,
+                                          acc, sigma2, valid ? slot : 0);
         else
             bad = detect_group<NL, ND, NR>(hr, hg, Yt + grp * nd * ys, Ht + grp * ht, hs, nb, nd, nl,
-                                           g.sigma2 ? g.loading : g.load, i, src0, acc, g.sigma2, valid ? slot : 0, ys);
+                                           sigma2 ? g.loading : g.load, i, src0, acc, sigma2, valid ? slot : 0, ys);
         if (valid && bad && i == 0) {
             atomicAdd(&status[1], 1u);
             atomicMin(&status[2], (unsigned)my_sc);
@@ -381,8 +383,8 @@ mmse_kernel(const __grid_constant__ MmseArgs g, long long total_sc, const float2
 }
 
 template <int NL, int ND, int WARPS, int NB>
-cudaError_t launch_nl(const MmseArgs &a, long long total_sc, const float2 *H, const float2 *beam, float2 *xhat,
-                      uint8_t *bits, uint32_t *status, cudaStream_t st) {
+cudaError_t launch_nl(const MmseArgs &a, long long total_sc, const float2 *H, const float2 *beam, const float2 *ls,
+                      const float *sigma2, float2 *xhat, uint8_t *bits, uint32_t *status, cudaStream_t st) {
     constexpr int SPW = 32 / NL;
     const size_t smem = (size_t)WARPS * warp_smem_bytes<NL>(a.n_beams, ND > 0 ? ND : a.n_det) + (NB > 0 ? 8 * WARPS : 0);
     const long long per_cta = (long long)WARPS * SPW;
@@ -393,7 +395,7 @@ cudaError_t launch_nl(const MmseArgs &a, long long total_sc, const float2 *H, co
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    k<<<(unsigned)grid, WARPS * 32, smem, st>>>(a, total_sc, H, beam, xhat, bits, status);
+    launch_chained(a.chained, k, dim3((unsigned)grid), dim3(WARPS * 32), smem, st, a, total_sc, H, beam, ls, sigma2, xhat, bits, status);
     return cudaGetLastError();
 }
 
@@ -405,33 +407,33 @@ constexpr size_t kMmseSmemMax = 227 * 1024;
 // data symbols or per symbol); anything else at run time. The defaults fit every supported shape (at most 64
 // beams and 12 data symbols: 120 KB for a 2-layer warp of 16 subcarriers).
 template <int NL, int NB>
-cudaError_t launch_w(const MmseArgs &a, long long total_sc, const float2 *H, const float2 *beam, float2 *xhat,
-                     uint8_t *bits, uint32_t *status, cudaStream_t st) {
+cudaError_t launch_w(const MmseArgs &a, long long total_sc, const float2 *H, const float2 *beam, const float2 *ls,
+                     const float *sigma2, float2 *xhat, uint8_t *bits, uint32_t *status, cudaStream_t st) {
     constexpr int W = mmse_default_warps<NL>();
     const bool fits = (size_t)a.warps * warp_smem_bytes<NL>(a.n_beams, a.n_det) <= kMmseSmemMax;
-    if (a.n_det == 12 && fits && a.warps == 1) return launch_nl<NL, 12, 1, NB>(a, total_sc, H, beam, xhat, bits, status, st);
-    if (a.n_det == 12 && fits && a.warps == 2) return launch_nl<NL, 12, 2, NB>(a, total_sc, H, beam, xhat, bits, status, st);
-    if (a.n_det == 12 && fits && a.warps == 4) return launch_nl<NL, 12, 4, NB>(a, total_sc, H, beam, xhat, bits, status, st);
-    if (a.n_det == 12 && fits && a.warps == 8) return launch_nl<NL, 12, 8, NB>(a, total_sc, H, beam, xhat, bits, status, st);
-    if (a.n_det == 12) return launch_nl<NL, 12, W, NB>(a, total_sc, H, beam, xhat, bits, status, st);
-    if (a.n_det == 4) return launch_nl<NL, 4, W, NB>(a, total_sc, H, beam, xhat, bits, status, st);
-    if (a.n_det == 1) return launch_nl<NL, 1, W, NB>(a, total_sc, H, beam, xhat, bits, status, st);
-    return launch_nl<NL, 0, W, 0>(a, total_sc, H, beam, xhat, bits, status, st);
+    if (a.n_det == 12 && fits && a.warps == 1) return launch_nl<NL, 12, 1, NB>(a, total_sc, H, beam, ls, sigma2, xhat, bits, status, st);
+    if (a.n_det == 12 && fits && a.warps == 2) return launch_nl<NL, 12, 2, NB>(a, total_sc, H, beam, ls, sigma2, xhat, bits, status, st);
+    if (a.n_det == 12 && fits && a.warps == 4) return launch_nl<NL, 12, 4, NB>(a, total_sc, H, beam, ls, sigma2, xhat, bits, status, st);
+    if (a.n_det == 12 && fits && a.warps == 8) return launch_nl<NL, 12, 8, NB>(a, total_sc, H, beam, ls, sigma2, xhat, bits, status, st);
+    if (a.n_det == 12) return launch_nl<NL, 12, W, NB>(a, total_sc, H, beam, ls, sigma2, xhat, bits, status, st);
+    if (a.n_det == 4) return launch_nl<NL, 4, W, NB>(a, total_sc, H, beam, ls, sigma2, xhat, bits, status, st);
+    if (a.n_det == 1) return launch_nl<NL, 1, W, NB>(a, total_sc, H, beam, ls, sigma2, xhat, bits, status, st);
+    return launch_nl<NL, 0, W, 0>(a, total_sc, H, beam, ls, sigma2, xhat, bits, status, st);
 }
 
 // The 16- and 32-layer classes are also compiled for 32 and 64 beams.
 template <int NL>
-cudaError_t launch_nd(const MmseArgs &a, long long total_sc, const float2 *H, const float2 *beam, float2 *xhat,
-                      uint8_t *bits, uint32_t *status, cudaStream_t st) {
+cudaError_t launch_nd(const MmseArgs &a, long long total_sc, const float2 *H, const float2 *beam, const float2 *ls,
+                      const float *sigma2, float2 *xhat, uint8_t *bits, uint32_t *status, cudaStream_t st) {
     if constexpr (NL >= 16) {
         // the beam-count instances stage by bulk copies: 16-byte aligned rows
         const bool aligned = reinterpret_cast<uintptr_t>(H) % 16 == 0 && reinterpret_cast<uintptr_t>(beam) % 16 == 0 &&
-                             reinterpret_cast<uintptr_t>(a.ls) % 16 == 0;
-        if (aligned && a.n_beams == 32) return launch_w<NL, 32>(a, total_sc, H, beam, xhat, bits, status, st);
-        if (aligned && a.n_beams == 64) return launch_w<NL, 64>(a, total_sc, H, beam, xhat, bits, status, st);
+                             reinterpret_cast<uintptr_t>(ls) % 16 == 0;
+        if (aligned && a.n_beams == 32) return launch_w<NL, 32>(a, total_sc, H, beam, ls, sigma2, xhat, bits, status, st);
+        if (aligned && a.n_beams == 64) return launch_w<NL, 64>(a, total_sc, H, beam, ls, sigma2, xhat, bits, status, st);
     }
-    if (a.ls) return cudaErrorNotSupported;   // only the beam-count instances interpolate while staging
-    return launch_w<NL, 0>(a, total_sc, H, beam, xhat, bits, status, st);
+    if (ls) return cudaErrorNotSupported;   // only the beam-count instances interpolate while staging
+    return launch_w<NL, 0>(a, total_sc, H, beam, ls, sigma2, xhat, bits, status, st);
 }
 
 // Warps per CTA that a.warps may select for the 12-symbol kernels of a layer class with n_beams beams (the
@@ -452,10 +454,13 @@ int mmse_warp_choices(int n_beams, int *out) {
 // Launch of one layer class (separate translation units, compiled in parallel): NL = 2, 4 or 8 in
 // mmse_small.cu, 16 in mmse_nl16.cu, 32 in mmse_nl32.cu.
 cudaError_t mmse_launch_class(int nl_class, const mmse_detail::MmseArgs &a, long long total_sc, const float2 *H,
-                              const float2 *beam, float2 *xhat, uint8_t *bits, uint32_t *status, cudaStream_t st);
+                              const float2 *beam, const float2 *ls, const float *sigma2, float2 *xhat,
+                                uint8_t *bits, uint32_t *status, cudaStream_t st);
 cudaError_t mmse_launch_class16(const mmse_detail::MmseArgs &a, long long total_sc, const float2 *H,
-                                const float2 *beam, float2 *xhat, uint8_t *bits, uint32_t *status, cudaStream_t st);
+                                const float2 *beam, const float2 *ls, const float *sigma2, float2 *xhat,
+                                uint8_t *bits, uint32_t *status, cudaStream_t st);
 cudaError_t mmse_launch_class32(const mmse_detail::MmseArgs &a, long long total_sc, const float2 *H,
-                                const float2 *beam, float2 *xhat, uint8_t *bits, uint32_t *status, cudaStream_t st);
+                                const float2 *beam, const float2 *ls, const float *sigma2, float2 *xhat,
+                                uint8_t *bits, uint32_t *status, cudaStream_t st);
 
 }  // namespace pusch

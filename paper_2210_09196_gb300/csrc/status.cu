@@ -15,6 +15,8 @@ namespace pusch {
 namespace {
 
 __global__ void status_fold_kernel(uint32_t *status, uint32_t *err) {
+    chain_wait(status, err);
+    chain_go();
     const uint32_t e = *err;
     if (e != 0u) {
         status[0] |= (uint32_t)PUSCH_STATUS_TIMEOUT;
@@ -44,7 +46,7 @@ pusch_status sfail(pusch_status st, const char *msg) {
 }  // namespace
 
 cudaError_t launch_status_fold(uint32_t *status, uint32_t *err, cudaStream_t st) {
-    status_fold_kernel<<<1, 1, 0, st>>>(status, err);
+    launch_chained(true, status_fold_kernel, dim3(1), dim3(1), 0, st, status, err);
     return cudaGetLastError();
 }
 
