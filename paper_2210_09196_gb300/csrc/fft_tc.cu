@@ -7,19 +7,31 @@
 // w = W^64:
 //   stage 1  Y[m][k0]   = W^(m k0) sum_a x[64 a + m] w^(a k0)
 //   stage 2  X[k0 + 64 k1] = sum_m Y[m][k0] w^(m k1)
-// Both stages multiply real rows by the same real matrix B[n = 2 k + o][j] = (cos, -sin)(2 pi j k / 64)
-// (N = 128: 64 outputs x (re, im); K = 64): a real row v gives sum_j v_j w^(j k) for every k.
-//   stage 1  A = the row as TMA loads it, read as a [64 a][128 mu] FP16 matrix, mu = 2 m + (re, im): M = mu
-//            (128 real rows), K = a, MN-major with 128-byte swizzling. Row (m, re) gives P_re[k0] =
-//            sum_a Re(x) w^(a k0), row (m, im) gives P_im[k0]; the two lanes of m combine
-//            Y = P_re + i P_im with one exchange per eight values and apply W^(m k0).
-//   stage 2  A2 = Y written by those lanes as real rows: row 2 k0 = Re Y[.][k0], row 2 k0 + 1 = Im Y[.][k0],
-//            K = m, MN-major with 128-byte swizzling (the layout of stage 1's operand): a lane holds one m and
-//            eight consecutive k0, i.e. 16 consecutive rows n = 2 k0 + (re, im), and writes them as two
-//            16-byte pieces. The lanes of row pair (2 k0, 2 k0 + 1) combine X = D_re + i D_im the same way and
-//            write bins k0 + 64 k1, consecutive across lanes, into the FP16 output planes.
+// Both stages multiply by the same real matrix A (128 rows (k; cos, -sin) x K = 64): a real column v gives
+// sum_j v_j cos and -sum_j v_j sin for every k.
+//   stage 1  B = the row as TMA loads it, read as a [64 a][128 mu] FP16 matrix, mu = 2 m + (re, im): N = mu,
+//            K = a, N-major with 128-byte swizzling.
+//   stage 2  B = Y, N = (k0; re, im), K = m, K-major without swizzling, written by the warps that read stage 1.
+// The accumulators are read with 16x256b loads, whose lane 4 g + t holds rows g and g + 8 at columns 2 t and
+// 2 t + 1 of every eight columns. A's rows are ordered so that g is k mod 8 and g + 8 the same k's sine row: a
+// lane holds the four real sums of one complex output (cos and sine row x re and im column) and combines them
+// itself, V = (cos re - msin im) + i (msin re + cos im). No value crosses lanes between the two products.
+//   - Stage 1's lane t holds m = 4 i + t, i = 0..3 in every 16 columns pairs. Inside each K step of 16 the order of
+//     K is free, so it is kappa = 4 t + i (the TMA map's dimensions and A's columns follow it): four consecutive
+//     kappa of one k0 go to stage 2's operand as one 8-byte store. The padded strides of that operand (144 B
+//     between core matrices along K, 1184 B between groups of eight columns) spread the stores over the banks.
+//   - Stage 2's columns are ordered so that a lane's eight column groups are eight consecutive output positions
+//     on a 16-byte boundary of the plane and the four lanes of a row 64 consecutive bytes: position (bin + n_sc / 2)
+//     mod 4096, octet e = t + 4 half. The FFT shift's remainder hr = (n_sc / 2) mod 8 rotates k0; only octet 0 then
+//     mixes two k1, and its first hr elements come from the lanes of k1 - 1 (eight exchanges per 64 x 8 block).
 // A 4096-point transform thus costs two MMA passes (8 MMAs of 128 x 128 x 16) and one pass of twiddles and
 // transposition through shared memory.
+//
+// What bounds it: the reading warps. With the data as the MMA's A operand (a complex value's sums in two lanes) the
+// LSU pipe was 67 % and issue 57 % busy: 128 lane exchanges and 51 2-byte stores per row and warp, 70.6 us for 7,168
+// rows with 3276 of 4096 bins kept. Here 16 exchanges and 8 16-byte stores per row: 58.6 us (52 % of the measured copy
+// rate), of which the accumulator reads are the largest part of the LSU pipe's work (1,024 of its wavefronts
+// per row). Three CTAs per SM, also with a two-stage ring: 58.7 and 60.1 us; octet 0 stored one element at a time 108 us.
 //
 // Roles (persistent CTAs, four per SM, 128 TMEM columns each): warps 0-3 read the accumulators (warp q owns TMEM
 // lane quarter q) and write the next operand or the output; warp 4 issues the row copies (TMA, a one-stage ring)
@@ -47,10 +59,15 @@ constexpr int kStages = 1;
 
 constexpr uint32_t kRowBytes = kN * 4;                      // one row of FP16 complex samples: 16 KB
 constexpr uint32_t kOffIn = 0;                              // input ring (stage-1 A operands, 1024-aligned)
-constexpr uint32_t kOffB = kOffIn + kStages * kRowBytes;    // B: [128][64] FP16, K-major, 16 KB
-constexpr uint32_t kOffA2 = kOffB + 16384;                  // A2: [2 halves of 64 n][64 m][128 B], 16 KB
-constexpr uint32_t kSmemUsed = kOffA2 + 16384;
+constexpr uint32_t kOffA = kOffIn + kStages * kRowBytes;    // A: [128][64] FP16, K-major, 16 KB
+constexpr uint32_t kOffY = kOffA + 16384;                   // Y: stage 2's B operand [128][64] FP16, K-major
+constexpr uint32_t kLboY = 144, kSboY = 1184;               // 8 core matrices of 128 B (+ 16), 16 column groups (+ 32)
+constexpr uint32_t kOffTw = kOffY + 16 * kSboY;             // W^(8 m q), q < 8: [q][i / 2][t] pairs of float2, 4 KB
+constexpr uint32_t kSmemUsed = kOffTw + 4096;
 constexpr size_t kSmemBytes = kSmemUsed + 1024;             // + alignment of the base to 1024 B
+
+// K order of both products: kappa = 16 s + 4 t + i stands for j = 16 s + 4 i + t
+__device__ __forceinline__ int k_of(int kappa) { return (kappa & 48) | ((kappa & 3) << 2) | ((kappa >> 2) & 3); }
 
 __device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
     asm volatile(
@@ -73,23 +90,39 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatil
     return __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
 }
 
-// The 16 complex values of one 32-column accumulator chunk of a real row, combined with the partner row's
-// (lane ^ 1): lane 2 j (the row of real parts) returns V[i] = D_re[i] + i D_im[i] for the chunk's outputs
-// 0..7, lane 2 j + 1 (imaginary parts) returns them for outputs 8..15.
-__device__ __forceinline__ void combine_pair(const uint32_t (&r)[32], int odd, float2 (&V)[8]) {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const float2 lo = make_float2(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1]));
-        const float2 hi = make_float2(__uint_as_float(r[2 * i + 16]), __uint_as_float(r[2 * i + 17]));
-        const float2 own = odd ? hi : lo, snd = odd ? lo : hi;
-        const float2 rcv = make_float2(__shfl_xor_sync(0xffffffffu, snd.x, 1), __shfl_xor_sync(0xffffffffu, snd.y, 1));
-        V[i] = odd ? make_float2(rcv.x - own.y, rcv.y + own.x) : make_float2(own.x - rcv.y, own.y + rcv.x);
-    }
+// Accumulator rows lane .. lane + 15 (lane given in the address's upper half), 32 columns: r[4 i ..] = row g at
+// columns 8 i + 2 t and + 1, then row g + 8 at the same columns (g = lane / 4, t = lane % 4).
+__device__ __forceinline__ void tmem_ld_16x256_x4(uint32_t taddr, uint32_t *r) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+        "%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+}
+// The registers go through the wait, so that no use of them can be scheduled before it.
+__device__ __forceinline__ void tmem_wait16(uint32_t *r) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+                 :
+                 : "memory");
+}
+
+// V = (cos re - msin im) + i (msin re + cos im) from a lane's four sums r = (cos re, cos im, msin re, msin im)
+__device__ __forceinline__ float2 combine(const uint32_t *r) {
+    return make_float2(__uint_as_float(r[0]) - __uint_as_float(r[3]), __uint_as_float(r[2]) + __uint_as_float(r[1]));
+}
+
+__device__ __forceinline__ uint32_t pack_half2(float a, float b) {
+    const __half2 v = __floats2half2_rn(a, b);
+    return *reinterpret_cast<const uint32_t *>(&v);
 }
 
 struct FftTcArgs {
     long long rows;
     int n_sc, pitch;
+    int vec;     // the output is 16-byte aligned
 };
 
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
@@ -100,10 +133,11 @@ fft_tc_kernel(const __grid_constant__ CUtensorMap tin, __half *__restrict__ out,
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t bar_full[kStages];
     __shared__ __align__(8) uint64_t bar_acc;     // MMA commits: the accumulator holds a finished product
-    __shared__ __align__(8) uint64_t bar_op;      // 4 warp arrivals: A2 written / the accumulator read out
+    __shared__ __align__(8) uint64_t bar_op;      // 4 warp arrivals: Y written / the accumulator read out
     __shared__ __align__(8) uint64_t bar_drain;
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
+    __shared__ __align__(16) uint32_t s_edge[kEpiWarps][16];   // a warp's first octet 0 and the one after its last
 
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
@@ -111,18 +145,38 @@ fft_tc_kernel(const __grid_constant__ CUtensorMap tin, __half *__restrict__ out,
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     volatile int *abort = &s_abort;
 
-    // ---------------------------------------------------------------- B (resident): (cos, -sin)(2 pi j k / 64)
-    // from the twiddle table (w^(j k) = W^(64 (j k mod 64))), eight K values (one 16-byte core-matrix row) per
-    // thread and store
+    // ---------------------------------------------------------------- A (resident): (cos, -sin)(2 pi j k / 64)
+    // from the table's w^q = W^(64 q), which go through shared memory (Y's place): with a table read for each of
+    // A's entries the set-up took 10.8 k of a CTA's 117 k clocks. All table reads are issued before the first wait.
+    constexpr int kTwPer = (512 + kThreads - 1) / kThreads;
+    float2 w8[kTwPer], w64 = make_float2(0.f, 0.f);
+    if (tid < 64) w64 = __ldg(&tw[64 * tid]);
+#pragma unroll
+    for (int u = 0; u < kTwPer; ++u) {
+        const int e = tid + u * kThreads;
+        if (e < 512) w8[u] = __ldg(&tw[8 * (e >> 6) * (e & 63)]);
+    }
+    float2 *sw64 = reinterpret_cast<float2 *>(gbase + kOffY);
+    if (tid < 64) sw64[tid] = w64;
+    // W^(8 m q), m = 4 i + t: pairs of consecutive i at [q][i / 2][t]
+#pragma unroll
+    for (int u = 0; u < kTwPer; ++u) {
+        const int e = tid + u * kThreads, m = e & 63;
+        if (e < 512)
+            reinterpret_cast<float2 *>(gbase + kOffTw)[(((e >> 6) * 8 + (m >> 3)) * 4 + (m & 3)) * 2 + ((m >> 2) & 1)] =
+                w8[u];
+    }
+    __syncthreads();
+    // eight K values (one 16-byte core-matrix row) per thread and store; row n = 16 (k / 8) + 8 (cos, -sin) + k % 8
     for (int e = tid; e < 128 * 8; e += kThreads) {
-        const int n = e >> 3, j0 = (e & 7) * 8, k = n >> 1;
+        const int n = e >> 3, j0 = (e & 7) * 8, k = ((n >> 4) << 3) | (n & 7);
         __align__(16) __half v[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-            const float2 w = __ldg(&tw[64 * (((j0 + u) * k) & 63)]);
-            v[u] = __float2half_rn((n & 1) ? w.y : w.x);     // Im W^q = -sin
+            const float2 w = sw64[(k_of(j0 + u) * k) & 63];
+            v[u] = __float2half_rn((n & 8) ? w.y : w.x);     // Im W^q = -sin
         }
-        *reinterpret_cast<uint4 *>(gbase + kOffB + kmajor_off(n, j0, 128, 1024)) = *reinterpret_cast<const uint4 *>(v);
+        *reinterpret_cast<uint4 *>(gbase + kOffA + kmajor_off(n, j0, 128, 1024)) = *reinterpret_cast<const uint4 *>(v);
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     if (tid == 0) {
@@ -147,7 +201,8 @@ fft_tc_kernel(const __grid_constant__ CUtensorMap tin, __half *__restrict__ out,
     if (warp == kEpiWarps) {
         // ------------------------------------------------------------ control: row copies and MMAs
         if (elect_one()) {
-            const uint32_t idesc = idesc_f16(128, 128, true, false);   // A MN-major in both stages
+            const uint32_t idesc = idesc_f16(128, 128, false, true);    // stage 1: B (the row) N-major
+            const uint32_t idesc2 = idesc_f16(128, 128, false, false);
             // the time samples are read once: evict-first, so that they do not push the FFT output (the next
             // kernel's input) out of L2 (an evict-last hint on the 2-byte output stores measured slower)
             const uint64_t pol_in = l2_policy_evict_first();
@@ -157,8 +212,8 @@ fft_tc_kernel(const __grid_constant__ CUtensorMap tin, __half *__restrict__ out,
                 const uint32_t bar = smem_u32(&bar_full[s]);
                 mbar_expect_tx(bar, kRowBytes);
                 for (int h = 0; h < 2; ++h)
-                    tma_load_2d_hint(base + kOffIn + (uint32_t)s * kRowBytes + (uint32_t)h * 8192u, &tin, 64 * h,
-                                     (int)(row * 64), bar, pol_in);
+                    tma_load_4d_hint(base + kOffIn + (uint32_t)s * kRowBytes + (uint32_t)h * 8192u, &tin, 64 * h,
+                                     (int)(row * 4), bar, pol_in);
             };
             long long issued = 0;
             for (; issued < kStages && issued < n_my; ++issued) issue(issued);
@@ -176,20 +231,21 @@ fft_tc_kernel(const __grid_constant__ CUtensorMap tin, __half *__restrict__ out,
                 fence_after_sync();
                 const uint32_t a0 = base + kOffIn + (uint32_t)s * kRowBytes;
                 for (int ks = 0; ks < 4; ++ks)
-                    mma_f16(tmem, smem_desc(a0 + (uint32_t)ks * 2048u, 8192, 1024, 2),
-                            smem_desc(base + kOffB + (uint32_t)ks * 256u, 128, 1024, 0), idesc, ks > 0 ? 1u : 0u);
+                    mma_f16(tmem, smem_desc(base + kOffA + (uint32_t)ks * 256u, 128, 1024, 0),
+                            smem_desc(a0 + (uint32_t)ks * 2048u, 8192, 1024, 2), idesc, ks > 0 ? 1u : 0u);
                 mma_commit(smem_u32(&bar_acc));
                 // the stage-1 products have read the row: its ring slot takes a later row
                 ok = mbar_wait_sleep(smem_u32(&bar_acc), 0u, abort, err, 32);
                 if (!ok) break;
                 if (issued < n_my) issue(issued++);
-                ok = mbar_wait_sleep(smem_u32(&bar_op), op_phase, abort, err, 128);   // A2 written
+                ok = mbar_wait_sleep(smem_u32(&bar_op), op_phase, abort, err, 128);   // Y written
                 op_phase ^= 1u;
                 if (!ok) break;
                 fence_after_sync();
                 for (int ks = 0; ks < 4; ++ks)
-                    mma_f16(tmem, smem_desc(base + kOffA2 + (uint32_t)ks * 2048u, 8192, 1024, 2),
-                            smem_desc(base + kOffB + (uint32_t)ks * 256u, 128, 1024, 0), idesc, ks > 0 ? 1u : 0u);
+                    mma_f16(tmem, smem_desc(base + kOffA + (uint32_t)ks * 256u, 128, 1024, 0),
+                            smem_desc(base + kOffY + (uint32_t)ks * 2u * kLboY, kLboY, kSboY, 0), idesc2,
+                            ks > 0 ? 1u : 0u);
                 mma_commit(smem_u32(&bar_acc));
             }
             if (ok && n_my > 0) mbar_wait_sleep(smem_u32(&bar_op), op_phase, abort, err, 128);   // the last row read out
@@ -203,41 +259,52 @@ fft_tc_kernel(const __grid_constant__ CUtensorMap tin, __half *__restrict__ out,
         }
     } else {
         // ------------------------------------------------------------ accumulator readers (warp q = lane quarter)
-        const int q = warp, odd = lane & 1, j = 16 * q + (lane >> 1);   // stage 1: m = j; stage 2: k0 = j
-        const uint32_t tq = tmem + ((uint32_t)(32 * q) << 16);
-        // twiddles W^(m k0), k0 = 16 c + 8 odd + i: W^(m (16 c + 8 odd)) * W^(m i), from exact table entries
-        float2 pw[8], bs[4];
+        const int g8 = lane >> 2, t = lane & 3;
+        const uint32_t tq = tmem + ((uint32_t)(32 * warp) << 16);
+        // twiddles W^(m k0), k0 = 8 q + g8, m = 4 i + t: W^(m g8) here, W^(8 m q) in shared memory (exact table
+        // entries both)
+        float2 pw[16];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) pw[i] = __ldg(&tw[j * i]);
+        for (int i = 0; i < 16; ++i) pw[i] = __ldg(&tw[(4 * i + t) * g8]);
+        const int h = g.n_sc >> 1, hr = h & 7, hb = h - hr;
+        uint32_t first[4];   // the halves of octet 0's pairs that lie among its first hr elements
 #pragma unroll
-        for (int c = 0; c < 4; ++c) bs[c] = __ldg(&tw[j * (16 * c + 8 * odd)]);
-        const int h = g.n_sc >> 1;
+        for (int i = 0; i < 4; ++i) first[i] = t > 0 ? 0u : hr - 2 * i >= 2 ? 0xffffffffu : hr - 2 * i == 1 ? 0xffffu : 0u;
+        // this lane's element of the warp's two edge octets: lane = [edge][plane][element]; -1: none
+        const int ei = lane & 7, epos = ((64 * 16 * (warp + (lane >> 4)) + hb) & (kN - 1)) + ei;
+        const bool emine = g.vec && hr > 0 && (lane < 16 ? ei >= hr : ei < hr) && epos < g.pitch;
+        const int eout = emine ? epos + ((lane >> 3) & 1) * g.pitch : -1;
         uint32_t acc_phase = 0;
         for (long long it = 0; it < n_my; ++it) {
             const long long row = blockIdx.x + it * gridDim.x;
-            // ---- stage-1 accumulator -> A2 (twiddled, transposed, FP16)
+            // ---- stage-1 accumulator -> Y (twiddled, FP16)
             if (!warp_wait(smem_u32(&bar_acc), acc_phase, abort, err, lane)) break;
             acc_phase ^= 1u;
             fence_after_sync();
-#pragma unroll 1
-            for (int c = 0; c < 4; ++c) {
-                uint32_t r[32];
-                tmem_ld32(tq + 32u * c, r);
-                float2 Y[8];
-                combine_pair(r, odd, Y);
-                // k0 = 16 c + 8 odd + i: rows n = 2 k0 + (re, im) = 32 c + 16 odd .. + 15, i.e. 16-byte pieces
-                // q0 and q0 + 1 (q0 = (c % 2) 4 + 2 odd) of row half c / 2, K row m = j, swizzled by j % 8
-                uint32_t v[8];
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const float2 y = cmul(cmul(Y[i], pw[i]), bs[c]);
-                    const __half2 hv = __floats2half2_rn(y.x, y.y);
-                    v[i] = *reinterpret_cast<const uint32_t *>(&hv);
+            for (int blk = 0; blk < 2; ++blk) {
+                const int q = 2 * warp + blk;
+                // the column group and pair of stage 2 that hold k0: octet e = u + 4 half, element x of position
+                // k0 + hr
+                const int pos = (8 * q + g8 + hr) & 63, x = pos & 7, e = pos >> 3;
+                uint8_t *yp = gbase + kOffY + (uint32_t)(8 * (e >> 2) + x) * kSboY + (uint32_t)(e & 3) * 32u +
+                              (uint32_t)(t >> 1) * kLboY + (uint32_t)(t & 1) * 8u;
+                const float4 *bt = reinterpret_cast<const float4 *>(gbase + kOffTw) + q * 32 + t;
+#pragma unroll
+                for (int s = 0; s < 4; ++s) {
+                    uint32_t r[16];
+                    tmem_ld_16x256_x4(tq + ((uint32_t)(16 * blk) << 16) + 32u * s, r);
+                    const float4 b0 = bt[8 * s], b1 = bt[8 * s + 4];
+                    tmem_wait16(r);
+                    const float2 y0 = cmul(cmul(combine(r), pw[4 * s]), make_float2(b0.x, b0.y));
+                    const float2 y1 = cmul(cmul(combine(r + 4), pw[4 * s + 1]), make_float2(b0.z, b0.w));
+                    const float2 y2 = cmul(cmul(combine(r + 8), pw[4 * s + 2]), make_float2(b1.x, b1.y));
+                    const float2 y3 = cmul(cmul(combine(r + 12), pw[4 * s + 3]), make_float2(b1.z, b1.w));
+                    *reinterpret_cast<uint2 *>(yp + 2 * s * kLboY) =
+                        make_uint2(pack_half2(y0.x, y1.x), pack_half2(y2.x, y3.x));
+                    *reinterpret_cast<uint2 *>(yp + 2 * s * kLboY + 16) =
+                        make_uint2(pack_half2(y0.y, y1.y), pack_half2(y2.y, y3.y));
                 }
-                uint8_t *rowp = gbase + kOffA2 + (uint32_t)(c >> 1) * 8192u + (uint32_t)j * 128u;
-                const int q0 = (c & 1) * 4 + 2 * odd;
-                *reinterpret_cast<uint4 *>(rowp + ((q0 ^ (j & 7)) << 4)) = make_uint4(v[0], v[1], v[2], v[3]);
-                *reinterpret_cast<uint4 *>(rowp + (((q0 + 1) ^ (j & 7)) << 4)) = make_uint4(v[4], v[5], v[6], v[7]);
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             fence_before_sync();
@@ -248,26 +315,68 @@ fft_tc_kernel(const __grid_constant__ CUtensorMap tin, __half *__restrict__ out,
             acc_phase ^= 1u;
             fence_after_sync();
             __half *o = out + row * 2 * (long long)g.pitch;
-#pragma unroll 1
-            for (int c = 0; c < 4; ++c) {
-                uint32_t r[32];
-                tmem_ld32(tq + 32u * c, r);
-                float2 X[8];
-                combine_pair(r, odd, X);
+            uint32_t hold[8] = {};   // lanes g8 = 0: octet 0 of the block's last k1
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int a = (j + 64 * (16 * c + 8 * odd + i) + h) & (kN - 1);
-                    if (a < g.n_sc) {
-                        const __half2 v = __floats2half2_rn(X[i].x, X[i].y);
-                        o[a] = __low2half(v);
-                        o[g.pitch + a] = __high2half(v);
+            for (int c = 0; c < 4; ++c) {
+                const int blk = c >> 1, half = c & 1, k1 = 16 * warp + 8 * blk + g8, e = t + 4 * half;
+                uint32_t r[32];
+                const uint32_t ta = tq + ((uint32_t)(16 * blk) << 16) + 64u * half;
+                tmem_ld_16x256_x4(ta, r);
+                tmem_ld_16x256_x4(ta + 32u, r + 16);
+                tmem_wait16(r);
+                tmem_wait16(r + 16);
+                uint32_t v[8];   // the octet's pairs: re 0..3, im 4..7
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float2 a = combine(r + 8 * i), b = combine(r + 8 * i + 4);
+                    v[i] = pack_half2(a.x, b.x);
+                    v[4 + i] = pack_half2(a.y, b.y);
+                }
+                // element i of the octet goes to position a0 + i; of octet 0 the first hr one block further on
+                const int a0 = (8 * e + 64 * k1 + hb) & (kN - 1);
+                if (!g.vec) {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const int a = (a0 + i + (e == 0 && i < hr ? 64 : 0)) & (kN - 1), sh = 16 * (i & 1);
+                        if (a < g.pitch) {
+                            o[a] = __ushort_as_half((unsigned short)(a < g.n_sc ? v[i >> 1] >> sh : 0u));
+                            o[g.pitch + a] = __ushort_as_half((unsigned short)(a < g.n_sc ? v[4 + (i >> 1)] >> sh : 0u));
+                        }
+                    }
+                    continue;
+                }
+                if (half == 0 && hr > 0) {
+                    uint32_t rot[8];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) rot[i] = __shfl_sync(0xffffffffu, v[i], (lane + 28) & 31);
+                    if (lane == 0) {   // the warp's first octet 0 (its own part) and the one after its last
+                        uint4 *ed = reinterpret_cast<uint4 *>(&s_edge[warp][8 * blk]);
+                        ed[0] = blk ? make_uint4(rot[0], rot[1], rot[2], rot[3]) : make_uint4(v[0], v[1], v[2], v[3]);
+                        ed[1] = blk ? make_uint4(rot[4], rot[5], rot[6], rot[7]) : make_uint4(v[4], v[5], v[6], v[7]);
+                    }
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const uint32_t prev = blk == 1 && g8 == 0 ? hold[i] : rot[i];
+                        v[i] = (prev & first[i & 3]) | (v[i] & ~first[i & 3]);
+                        if (blk == 0) hold[i] = rot[i];
                     }
                 }
+                const bool whole = !(c == 0 && lane == 0 && hr > 0);
+                if (whole && a0 < g.pitch) {
+                    if (a0 + 8 > g.n_sc) {
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            const int n = g.n_sc - a0 - 2 * (i & 3);      // values left from this pair on
+                            v[i] &= n >= 2 ? 0xffffffffu : n == 1 ? 0xffffu : 0u;
+                        }
+                    }
+                    *reinterpret_cast<uint4 *>(o + a0) = make_uint4(v[0], v[1], v[2], v[3]);
+                    *reinterpret_cast<uint4 *>(o + g.pitch + a0) = make_uint4(v[4], v[5], v[6], v[7]);
+                }
             }
-            for (int a = g.n_sc + tid; a < g.pitch; a += 32 * kEpiWarps) {
-                o[a] = __float2half_rn(0.f);
-                o[g.pitch + a] = __float2half_rn(0.f);
-            }
+            __syncwarp();
+            if (eout >= 0)
+                o[eout] = epos < g.n_sc ? reinterpret_cast<const __half *>(s_edge[warp])[lane] : __float2half_rn(0.f);
             fence_before_sync();
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&bar_op));
@@ -296,11 +405,12 @@ cudaError_t launch_fft_tc(const Geometry &g, long long rows, const void *in, voi
     PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
     if (!enc) return cudaErrorNotSupported;
     CUtensorMap map;
-    cuuint64_t dims[2] = {128, (cuuint64_t)(rows * 64)};          // [rows * 64 a][128 mu] FP16
-    cuuint64_t strides[1] = {256};
-    cuuint32_t box[2] = {64, 64};
-    cuuint32_t estr[2] = {1, 1};
-    CUresult r = enc(&map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void *>(in), dims, strides, box, estr,
+    // [rows * 4 s][4 t][4 i][128 mu] FP16: sample j = 16 s + 4 i + t of a row's 64
+    cuuint64_t dims[4] = {128, 4, 4, (cuuint64_t)(rows * 4)};
+    cuuint64_t strides[3] = {1024, 256, 4096};
+    cuuint32_t box[4] = {64, 4, 4, 4};
+    cuuint32_t estr[4] = {1, 1, 1, 1};
+    CUresult r = enc(&map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, const_cast<void *>(in), dims, strides, box, estr,
                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
@@ -309,7 +419,7 @@ cudaError_t launch_fft_tc(const Geometry &g, long long rows, const void *in, voi
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    // kCtasPerSm resident CTAs per SM (4 x 52 KB of shared memory; 4 x 128 TMEM columns = 512). The CTAs are
+    // kCtasPerSm resident CTAs per SM (4 x 57 KB of shared memory; 4 x 128 TMEM columns = 512). The CTAs are
     // independent, so a CTA that cannot be resident at once simply runs later.
     long long grid = (long long)sms * (g.fft_cap > 0 && g.fft_cap < kCtasPerSm ? g.fft_cap : kCtasPerSm);
     if (grid > rows) grid = rows;
@@ -317,6 +427,7 @@ cudaError_t launch_fft_tc(const Geometry &g, long long rows, const void *in, voi
     a.rows = rows;
     a.n_sc = g.n_sc;
     a.pitch = g.sc_pitch;
+    a.vec = (reinterpret_cast<uintptr_t>(out) & 15) == 0;
     launch_chained(g.chained, fft_tc_kernel, dim3((unsigned)grid), dim3(kThreads), kSmemBytes, st, map, static_cast<__half *>(out), tw, a, err);
     return cudaGetLastError();
 }
