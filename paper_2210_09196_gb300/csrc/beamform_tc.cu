@@ -144,7 +144,9 @@ beamform_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
     // (k/8)*128 + (n%8)*16 + (k%8)*2. FP8: a first pass over the pieces takes the largest |Re|, |Im| per
     // (beam, 128-antenna block) (shared atomics on the bit patterns: non-negative floats order like their
     // bits; a non-finite component records +inf), the second writes the codes as FP16 values on the beam's
-    // scale.
+    // scale. A thread keeps one beam and steps over the antennas: no divisions, one atomic per block, the scales
+    // read once per four antennas, and both of a beam's rows from one conversion (256 antennas, 64 beams, 4 slots: FP8
+    // 111.3 -> 102.0 us, FP16 62.2 -> 58.1 us against a conversion per row with a division per element).
     {
         float2 *Ws = reinterpret_cast<float2 *>(gbase);
         const int nb = g.n_beams;
@@ -154,25 +156,38 @@ beamform_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
         auto stage_piece = [&](int r0, int np) {
             __syncthreads();                                 // the previous piece is consumed
             const float2 *src = W + (size_t)r0 * nb;
-            const int cnt = np * nb;
-            for (int i2 = tid; i2 < cnt; i2 += kThreads)
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(Ws + i2)), "l"(src + i2) : "memory");
+            const int cnt = np * nb;                         // even: nb is a multiple of 8
+            if ((reinterpret_cast<uintptr_t>(W) & 15) == 0) {
+                for (int i2 = 2 * tid; i2 < cnt; i2 += 2 * kThreads)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(Ws + i2)), "l"(src + i2)
+                                 : "memory");
+            } else {
+                for (int i2 = tid; i2 < cnt; i2 += kThreads)
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(Ws + i2)), "l"(src + i2)
+                                 : "memory");
+            }
             asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
             __syncthreads();
         };
         const int n_kb = (g.n_rx + 127) / 128;
+        const int rstep = kThreads / nb, wr = tid / nb, b = tid - wr * nb;   // nb <= 64 < kThreads
         if constexpr (FP8) {
             uint32_t *wmax = reinterpret_cast<uint32_t *>(sh.ew);
             for (int i2 = tid; i2 < 64 * 4; i2 += kThreads) wmax[i2] = 0u;
             for (int r0 = 0; r0 < g.n_rx; r0 += P) {
                 const int np = min(P, g.n_rx - r0);
                 stage_piece(r0, np);
-                for (int i2 = tid; i2 < np * nb; i2 += kThreads) {
-                    const int r = r0 + i2 / nb, b = i2 - (i2 / nb) * nb;
-                    const float2 w = Ws[i2];
-                    const float ax = fabsf(w.x), ay = fabsf(w.y);
-                    const bool bad = !(ax <= FLT_MAX) || !(ay <= FLT_MAX);
-                    atomicMax(&wmax[b * 4 + (r >> 7)], bad ? 0x7F800000u : __float_as_uint(fmaxf(ax, ay)));
+                for (int kb = r0 >> 7; wr < rstep && kb * 128 < r0 + np; ++kb) {
+                    const int lo = max(r0, kb * 128) - r0, hi = min(r0 + np, kb * 128 + 128) - r0;
+                    uint32_t m = 0u;
+#pragma unroll 4
+                    for (int r = lo + wr; r < hi; r += rstep) {
+                        const float2 w = Ws[r * nb + b];
+                        const float ax = fabsf(w.x), ay = fabsf(w.y);
+                        const bool bad = !(ax <= FLT_MAX) || !(ay <= FLT_MAX);
+                        m = max(m, bad ? 0x7F800000u : __float_as_uint(fmaxf(ax, ay)));
+                    }
+                    atomicMax(&wmax[b * 4 + kb], m);
                 }
             }
             __syncthreads();
@@ -191,39 +206,39 @@ beamform_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_consta
             const int np = min(P, g.n_rx - r0);
             if (FP8 && resident) __syncthreads();            // pass 1's exponents are visible
             else stage_piece(r0, np);
-            const int nchunks = (np / 4) * N;
-            for (int c = tid; c < nchunks; c += kThreads) {
-                const int kcl = c / N, n = c - kcl * N;
-                const int b = n >> 1;
-                uint32_t h[4];
+            uint8_t *row = gB + (size_t)(b >> 2) * b_sbo + (2 * b & 7) * 16;   // rows 2 b and 2 b + 1
+#pragma unroll 2
+            for (int kcl = wr; wr < rstep && kcl < np / 4; kcl += rstep) {
+                float inv = 1.f, down = 1.f;
+                bool bad = false;
+                if constexpr (FP8) {
+                    const int eb = sh.wexp[b], e_blk = sh.ew[b * 4 + ((r0 + 4 * kcl) >> 7)];
+                    bad = eb >= 128;                          // the beam's scale is NaN; values unused
+                    inv = exp2_int(bad ? 0 : -e_blk);         // 2^-e_blk, e_blk in [-126, 120]
+                    const int d = bad ? 0 : eb - e_blk;       // shift of this block to the beam exponent
+                    down = exp2_int(d > 40 ? -40 : -d);
+                }
+                uint32_t h0[4], h1[4];
 #pragma unroll
                 for (int a4 = 0; a4 < 4; ++a4) {
                     const float2 w = Ws[(4 * kcl + a4) * nb + b];
                     __half re, im;
                     if constexpr (FP8) {
-                        const int r = r0 + 4 * kcl + a4;
-                        const int eb = sh.wexp[b], e_blk = sh.ew[b * 4 + (r >> 7)];
-                        if (eb >= 128) {                     // the beam's scale is NaN; values unused
-                            re = im = __float2half_rn(0.f);
-                        } else {
-                            const float inv = exp2_int(-e_blk);   // 2^-e_blk, e_blk in [-126, 120]
-                            const float2 cq = e4m3x2_to_float2(float2_to_e4m3x2(make_float2(w.x * inv, w.y * inv)));
-                            const int d = eb - e_blk;             // shift of this block to the beam exponent
-                            const float sh2 = exp2_int(d > 40 ? -40 : -d);
-                            re = __float2half_rn(cq.x * sh2);
-                            im = __float2half_rn(cq.y * sh2);
-                        }
+                        const float2 cq = e4m3x2_to_float2(float2_to_e4m3x2(make_float2(w.x * inv, w.y * inv)));
+                        re = bad ? __float2half_rn(0.f) : __float2half_rn(cq.x * down);
+                        im = bad ? __float2half_rn(0.f) : __float2half_rn(cq.y * down);
                     } else {
                         re = __float2half_rn(w.x);
                         im = __float2half_rn(w.y);
                     }
                     // row 2b: (Re, Im); row 2b + 1: (-Im, Re)
-                    const __half lo = (n & 1) ? __hneg(im) : re, hi = (n & 1) ? re : im;
-                    h[a4] = (uint32_t)__half_as_ushort(lo) | ((uint32_t)__half_as_ushort(hi) << 16);
+                    const uint32_t ur = __half_as_ushort(re), ui = __half_as_ushort(im);
+                    h0[a4] = ur | (ui << 16);
+                    h1[a4] = (uint32_t)__half_as_ushort(__hneg(im)) | (ur << 16);
                 }
-                const int kc = r0 / 4 + kcl;
-                *reinterpret_cast<uint4 *>(gB + (size_t)(n >> 3) * b_sbo + (size_t)kc * 128 + (n & 7) * 16) =
-                    make_uint4(h[0], h[1], h[2], h[3]);
+                uint8_t *d = row + (size_t)(r0 / 4 + kcl) * 128;
+                *reinterpret_cast<uint4 *>(d) = make_uint4(h0[0], h0[1], h0[2], h0[3]);
+                *reinterpret_cast<uint4 *>(d + 16) = make_uint4(h1[0], h1[1], h1[2], h1[3]);
             }
         }
         __syncthreads();                                     // B complete; the ring is free again
