@@ -105,12 +105,16 @@ __device__ __forceinline__ float block_sum(float v, float *red) {
 }
 
 // grid[gi][ch][j][a] (bf16) = v_j[a] / scale with scale = rms over the grid; gi = (slot * L + l) * B + b.
+// The layer's LS values are formed once, in shared memory (n_pil of them per symbol; 0: they do not fit, and every
+// subcarrier forms its own). Formed per subcarrier and pass, eight loads a beam row apart and eight reciprocals each
+// bounded the kernel: one slot's estimate (512 grids of 3276, a pilot in 16) took 273 us, 245 so.
 __global__ void __launch_bounds__(256)
-ls_grid_kernel(GridArgs g, const float2 *__restrict__ beam, const float2 *__restrict__ pilots,
+ls_grid_kernel(GridArgs g, int smem_pilots, const float2 *__restrict__ beam, const float2 *__restrict__ pilots,
                __nv_bfloat16 *__restrict__ grid, float *__restrict__ scale) {
     chain_wait(beam, pilots, grid, scale);
     chain_go();
     __shared__ float red[32];
+    extern __shared__ float2 s_ls[];             // [2][n_pil]
     const long long gi = blockIdx.x;
     const int b = (int)(gi % g.n_beams);
     const long long sl_l = gi / g.n_beams;
@@ -121,10 +125,34 @@ ls_grid_kernel(GridArgs g, const float2 *__restrict__ beam, const float2 *__rest
     const float2 *p0 = pilots + (slot * g.n_layers + l) * 2LL * g.n_sc;
     const float2 *p1 = p0 + g.n_sc;
     const int port = g.port[l];
+    const int n_pil = smem_pilots ? (g.n_sc - 1 - port) / g.comb + 1 : 0;
+    for (int k = threadIdx.x; k < n_pil; k += blockDim.x) {
+        const int q = port + k * g.comb;
+        s_ls[k] = cmul(__ldg(&y0[(long long)q * g.n_beams]), pilot_inverse(__ldg(&p0[q])));
+        s_ls[n_pil + k] = cmul(__ldg(&y1[(long long)q * g.n_beams]), pilot_inverse(__ldg(&p1[q])));
+    }
+    __syncthreads();
+    auto values = [&](int a, float2 &v0, float2 &v1) {
+        if (n_pil == 0) {
+            v0 = grid_value(g, y0, p0, a, port);
+            v1 = grid_value(g, y1, p1, a, port);
+            return;
+        }
+        const int k = a <= port ? 0 : min((a - port) / g.comb, n_pil - 1), lo = port + k * g.comb;
+        v0 = s_ls[k];
+        v1 = s_ls[n_pil + k];
+        if (a > lo && k + 1 < n_pil) {
+            const float w = interp_weight(a, lo, lo + g.comb);
+            v0 = interp(v0, s_ls[k + 1], w);
+            v1 = interp(v1, s_ls[n_pil + k + 1], w);
+        }
+    };
     float ss = 0.f;
     for (int a = threadIdx.x; a < g.n_sc; a += blockDim.x) {
-        const float2 v0 = grid_value(g, y0, p0, a, port), v1 = grid_value(g, y1, p1, a, port);
-        ss += v0.x * v0.x + v0.y * v0.y + v1.x * v1.x + v1.y * v1.y;
+        float2 v0, v1;
+        values(a, v0, v1);
+        // the contraction is written out: another one moves the scale by an ulp and with it a BF16 rounding now and then
+        ss += fmaf(v1.y, v1.y, fmaf(v1.x, v1.x, fmaf(v0.x, v0.x, __fmul_rn(v0.y, v0.y))));
     }
     const float tot = block_sum(ss, red);
     const float sc = sqrtf(tot / (2.f * g.n_sc)) + 1e-30f;
@@ -132,7 +160,8 @@ ls_grid_kernel(GridArgs g, const float2 *__restrict__ beam, const float2 *__rest
     if (threadIdx.x == 0) scale[gi] = sc;
     __nv_bfloat16 *o = grid + gi * 4LL * g.n_sc;  // [2 ch][2 rows][n_sc]
     for (int a = threadIdx.x; a < g.n_sc; a += blockDim.x) {
-        const float2 v0 = grid_value(g, y0, p0, a, port), v1 = grid_value(g, y1, p1, a, port);
+        float2 v0, v1;
+        values(a, v0, v1);
         o[0 * g.n_sc + a] = __float2bfloat16_rn(v0.x * inv);
         o[1 * g.n_sc + a] = __float2bfloat16_rn(v1.x * inv);
         o[2 * g.n_sc + a] = __float2bfloat16_rn(v0.y * inv);
@@ -221,7 +250,10 @@ cudaError_t launch_ls_grid(const Geometry &g, int n_slots, const float2 *beam, c
     const long long grids = (long long)n_slots * g.n_layers * g.n_beams;
     if (grids == 0) return cudaSuccess;
     if (grids > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    launch_chained(true, ls_grid_kernel, dim3((unsigned)grids), dim3(256), 0, st, grid_args(g), beam, pilots, grid, scale);
+    const size_t bytes = ((size_t)(g.n_sc - 1) / g.comb + 1) * 2 * sizeof(float2);   // of the port with most pilots
+    const int fits = bytes <= 47 * 1024;
+    launch_chained(true, ls_grid_kernel, dim3((unsigned)grids), dim3(256), fits ? bytes : 0, st, grid_args(g), fits, beam,
+                   pilots, grid, scale);
     return cudaGetLastError();
 }
 
