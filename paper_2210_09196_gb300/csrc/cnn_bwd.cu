@@ -201,7 +201,10 @@ cnn_bwd_mid_kernel(BwdArgs g, const float *__restrict__ gout, const __nv_bfloat1
             for (int c = 0; c < 8; ++c)
                 av[j][c] = on ? __bfloat16_as_ushort(__ldg(ap + (long long)(2 * c) * g.w + 32 * j)) : (uint16_t)0;
         }
-        if (done) wait(bar_p, (done - 1) & 1u);                            // the last tile's operands are free
+        if (done) {
+            wait(bar_p, (done - 1) & 1u);                                  // the last tile's products have read their operands
+            ctx_sync(ctx);                                                 // and all warps its activations, the ReLU mask
+        }
         // ---- G in three parts
 #pragma unroll
         for (int i = 0; i < kBufRows / 16; ++i) {
