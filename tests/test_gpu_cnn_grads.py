@@ -6,7 +6,10 @@ wrong by its whole value.
 
 Tolerance: an input gradient is a sum of at most 192 products, in at most 36 truncated tensor-core steps (2^-23 of the
 running sum each) or 12 FMAs, of operands split to 2^-24 of themselves; with 48 * 2^-23 < 6e-6 of the sum of the products'
-magnitudes for each of the layers so far."""
+magnitudes for each of the layers so far. Truncation shrinks: half of a unit in the last place (2^-25 to 2^-24 of the
+sum) is lost on average in each step that meets a sum of full size. With the parts of the split operand taken smallest
+first these are 12 steps a layer, 12 * 2^-25 = 3.6e-7 of the norm where a step loses as little as it can (36 steps:
+1.1e-6)."""
 import numpy as np
 import pytest
 import torch
@@ -99,3 +102,16 @@ def test_input_gradients_with_several_tiles_per_cta(n, w):
             got = where.reshape(n, w, 2, 32).permute(0, 3, 2, 1).double()
             off = (got - g).abs()
             assert bool((off <= 6e-6 * (4 - k) * mag).all()), (k, float((off / mag.clamp(min=1e-300)).max()))
+
+
+def test_input_gradients_shrink_by_the_steps_of_the_largest_part():
+    n, w = 64, 96
+    c = inputs(n, w, 5)
+    _, _, work = backward(c)
+    P = layers(c["p"].double())
+    g = 2.0 * (c["y"].double() - c["target"].double()) / (4.0 * n * w)
+    for k, where in ((3, None), (2, work[0]), (1, work[1])):
+        g = input_grad(g, P[k][0], DIL[k]) * (c["acts"][k - 1] > 0)
+        if where is not None:
+            got = where.reshape(n, w, 2, 32).permute(0, 3, 2, 1).double()
+            assert float((got - g).norm() / g.norm()) < 3.6e-7 * (3 - k), k
