@@ -18,9 +18,12 @@
 //                    12 steps of the largest part should meet a sum of full size (largest first: g2 off by 8.1e-7 of its
 //                    norm, g1 by 1.7e-6; smallest first: 1.2e-7 and 2.0e-7).
 //   weight gradient  P[(part, h, co)][(kw, r, ci)] = sum_x G_part[(h, co)][x] A[(r, ci)][x + (kw - 1) dil]: the same
-//                    shared-memory rows read as MN-major operands, K = x. M = 128 holds the two upper parts, then the
-//                    lower part beside 64 rows of zeros; N = 192 holds the three taps, whose operand blocks lie dil rows
-//                    apart: 16 MMAs of 80 clocks. P stays in TMEM for all tiles of a CTA.
+//                    shared-memory rows read as MN-major operands, K = x. M = 128 holds 64 rows of zeros beside the lowest
+//                    part, then the two upper parts; N = 192 holds the three taps, whose operand blocks lie dil rows
+//                    apart: 16 MMAs of 80 clocks. P is formed anew in every tile and added up over the CTA's tiles in FP32
+//                    in shared memory: a sum that stayed in TMEM lost some 1.1e-7 of itself per tile to the truncation
+//                    (3.6e-6 at 4096 grids x 256, 1.3e-5 at 12288; now 3e-8, and the whole error is below that of rounded
+//                    FP32 sums of all products).
 // Two tiles are in flight per CTA (one CTA per SM), 256 threads each. Activations arrive in 2-byte loads along the
 // subcarriers (the caller's layout, any width) and go to shared memory channels-last.
 // Measured (GB300, a step of 1024 grids x 256): out 41, mid 93 each, in 21 us; on FP32 FMAs (weights gradient: one thread
@@ -95,8 +98,10 @@ __device__ __forceinline__ void store2(float *p, float a, float b, int vec) {
 constexpr int kHaloR = 16, kBufRows = kTile + 2 * kHaloR;
 constexpr uint32_t kPartBytes = kBufRows * 128;
 constexpr int kCtx = 2, kCtxThreads = 256, kMidThreads = kCtx * kCtxThreads;
-constexpr uint32_t kOffCtx = 24576, kCtxBytes = 4 * kPartBytes, kOffZero = kOffCtx + kCtx * kCtxBytes;
-constexpr size_t kMidSmem = 1024 + kOffZero + (kTile + kHaloR) * 128;
+// weights, 64 x 16 zeros, per context three parts of G and the activations, the CTA's weight gradient
+constexpr uint32_t kOffZero = 24576, kZeroBytes = 16 * 128, kOffCtx = kOffZero + kZeroBytes, kCtxBytes = 4 * kPartBytes;
+constexpr uint32_t kOffAcc = kOffCtx + kCtx * kCtxBytes;
+constexpr size_t kMidSmem = 1024 + kOffAcc + 9 * 1024 * 4;
 constexpr int kCtxCols = 256;     // TMEM: 64 columns of D, 192 of P
 
 // kind::f16 with BF16 operands, F32 accumulator, M = 128
@@ -118,6 +123,25 @@ __device__ __forceinline__ float2 minus_bf16(float2 v, uint32_t u) {
     return make_float2(v.x - __uint_as_float(u << 16), v.y - __uint_as_float(u & 0xffff0000u));
 }
 
+// Mutual exclusion of a CTA's contexts, by one thread of each; bounded as the waits on barriers are.
+__device__ __forceinline__ void lock_acquire(int *lock, volatile int *abort, uint32_t *err) {
+    const uint64_t deadline = globaltimer() + kWaitNs;
+    while (atomicCAS(lock, 0, 1) != 0) {
+        if (*abort) break;
+        if (globaltimer() > deadline) {
+            *abort = 1;
+            if (err) atomicOr(err, kErrTensorWait);
+            break;
+        }
+        __nanosleep(32);
+    }
+    __threadfence_block();
+}
+__device__ __forceinline__ void lock_release(int *lock) {
+    __threadfence_block();
+    atomicExch(lock, 0);
+}
+
 __global__ void __launch_bounds__(kMidThreads, 1)
 cnn_bwd_mid_kernel(BwdArgs g, const float *__restrict__ gout, const __nv_bfloat16 *__restrict__ acts,
                    const __nv_bfloat16 *__restrict__ W, float *__restrict__ gin, float *__restrict__ dW,
@@ -126,7 +150,7 @@ cnn_bwd_mid_kernel(BwdArgs g, const float *__restrict__ gout, const __nv_bfloat1
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t bar_d[kCtx], bar_p[kCtx];
     __shared__ uint32_t s_tmem;
-    __shared__ int s_abort;
+    __shared__ int s_abort, s_lock;
     __shared__ float s_db[32];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
@@ -134,7 +158,7 @@ cnn_bwd_mid_kernel(BwdArgs g, const float *__restrict__ gout, const __nv_bfloat1
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     volatile int *abort = &s_abort;
 
-    // B_kw[(r, ci)][(h, co)] = W[co][ci][r - h + 1][kw]; zeros beside the lower part
+    // B_kw[(r, ci)][(h, co)] = W[co][ci][r - h + 1][kw]; zeros beside the lowest part
     for (int i = tid; i < 32 * 32 * 9; i += kMidThreads) {
         const int co = i / 288, rem = i - co * 288, ci = rem / 9, kk = rem - ci * 9, kh = kk / 3, kw = kk - kh * 3;
         const __nv_bfloat16 v = W[i];
@@ -145,8 +169,9 @@ cnn_bwd_mid_kernel(BwdArgs g, const float *__restrict__ gout, const __nv_bfloat1
                 *reinterpret_cast<__nv_bfloat16 *>(gb + kw * 8192 + sw128(r * 32 + ci, h * 32 + co)) = v;
         }
     }
-    for (int i = tid; i < (kTile + kHaloR) * 8; i += kMidThreads)
-        reinterpret_cast<uint4 *>(gb + kOffZero)[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (tid < (int)kZeroBytes / 16) reinterpret_cast<uint4 *>(gb + kOffZero)[tid] = make_uint4(0u, 0u, 0u, 0u);
+    float *acc = reinterpret_cast<float *>(gb + kOffAcc);                  // [kh * 3 + kw][ci][co]
+    for (int i = tid; i < 9 * 1024; i += kMidThreads) acc[i] = 0.f;
     if (tid < 32) s_db[tid] = 0.f;
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     if (tid == 0) {
@@ -156,6 +181,7 @@ cnn_bwd_mid_kernel(BwdArgs g, const float *__restrict__ gout, const __nv_bfloat1
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         s_abort = 0;
+        s_lock = 0;
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
@@ -178,11 +204,39 @@ cnn_bwd_mid_kernel(BwdArgs g, const float *__restrict__ gout, const __nv_bfloat1
         fence_after_sync();
     };
 
+    // P of this context's tile -> acc, by all of the context's threads once the products have completed. A weight gets
+    // terms from four lane quarters q = (part, h) and two grid rows r: in each of four phases the quarters take different
+    // taps, and a quarter's two warps different r, so that no two threads add to the same word (with atomics the
+    // backward pass of 1024 grids x 256 took 315 us, so it takes 254, as with one sum over all tiles).
+    auto add_p = [&]() {
+        if (t8 == 0) lock_acquire(&s_lock, abort, err);
+        ctx_sync(ctx);
+        const int q = w8 & 3, h = q & 1, r = w8 >> 2;
+#pragma unroll 1
+        for (int f = 0; f < 4; ++f) {
+            const int kw = (q + f) & 3;
+            if (kw < 3) {
+                float v[32];                                               // 32 columns: tap kw, grid row r
+                tmem_ld32_nowait(tmP + quarter + 64u * kw + 32u * r, reinterpret_cast<uint32_t(&)[32]>(v));
+                tmem_wait_ld();
+                float *o = acc + ((r - h + 1) * 3 + kw) * 1024 + lane;     // lane: co
+#pragma unroll
+                for (int ci = 0; ci < 32; ++ci) o[ci * 32] += v[ci];
+            }
+            ctx_sync(ctx);
+        }
+        if (t8 == 0) lock_release(&s_lock);
+        fence_before_sync();
+    };
     const int ch4 = t8 & 15;                                               // this thread's channels 4 ch4 .. + 3 of G
     float4 dbs = make_float4(0.f, 0.f, 0.f, 0.f);
     uint32_t done = 0;                                                     // tiles of this context so far
     for (int t = blockIdx.x + ctx * gridDim.x; t < g.tiles; t += kCtx * gridDim.x, ++done) {
         const int gi = t / g.tiles_per_grid, x0 = (t - gi * g.tiles_per_grid) * kTile;
+        if (done) {                                                        // the last tile's products: its operands are free,
+            wait(bar_p, (done - 1) & 1u);                                  // and (the barriers in add_p) its activations,
+            add_p();                                                       // the ReLU mask, have been read by all warps
+        }
         // ---- all loads of the tile at once: G rows (t8 / 16) + 16 i, activations of channels 8 w8 .. + 7 of rows
         //      32 j + lane
         const float *gp = gout + (long long)gi * g.w * 64 + 4 * ch4;
@@ -203,10 +257,6 @@ cnn_bwd_mid_kernel(BwdArgs g, const float *__restrict__ gout, const __nv_bfloat1
 #pragma unroll
             for (int c = 0; c < 8; ++c)
                 av[j][c] = on ? __bfloat16_as_ushort(__ldg(ap + (long long)(2 * c) * g.w + 32 * j)) : (uint16_t)0;
-        }
-        if (done) {
-            wait(bar_p, (done - 1) & 1u);                                  // the last tile's products have read their operands
-            ctx_sync(ctx);                                                 // and all warps its activations, the ReLU mask
         }
         // ---- G in three parts
 #pragma unroll
@@ -256,15 +306,16 @@ cnn_bwd_mid_kernel(BwdArgs g, const float *__restrict__ gout, const __nv_bfloat1
             }
             mma_commit(smem_u32(&bar_d[ctx]));
             const uint64_t dG = smem_desc(cbase + kHaloR * 128u, kPartBytes, 1024, 2);
-            const uint64_t dL = smem_desc(cbase + 2 * kPartBytes + kHaloR * 128u, base + kOffZero - cbase - 2 * kPartBytes,
-                                          1024, 2);
+            // zeros, then the lowest part: the block of zeros is the same in every step, the distance grows
+            const uint64_t dL = smem_desc(base + kOffZero, cbase + 2 * kPartBytes + kHaloR * 128u - (base + kOffZero), 1024, 2);
             const uint64_t dX = smem_desc(cbase + 3 * kPartBytes + (uint32_t)(kHaloR - g.dil) * 128u, (uint32_t)g.dil * 128u,
                                           1024, 2);
 #pragma unroll 1
-            for (int ks = 0; ks < kTile / 16; ++ks) {
-                mma<false>(tmP, dG + 128u * ks, dX + 128u * ks, idesc_bf16(192, true), (done > 0 || ks > 0) ? 1u : 0u);
-                mma<false>(tmP, dL + 128u * ks, dX + 128u * ks, idesc_bf16(192, true), 1u);
-            }
+            for (int ks = 0; ks < kTile / 16; ++ks)
+                mma<false>(tmP, dL + ((uint64_t)(128u * ks) << 16), dX + 128u * ks, idesc_bf16(192, true), ks > 0 ? 1u : 0u);
+#pragma unroll 1
+            for (int ks = 0; ks < kTile / 16; ++ks)
+                mma<false>(tmP, dG + 128u * ks, dX + 128u * ks, idesc_bf16(192, true), 1u);
             mma_commit(smem_u32(&bar_p[ctx]));
         }
         __syncwarp();
@@ -294,33 +345,16 @@ cnn_bwd_mid_kernel(BwdArgs g, const float *__restrict__ gout, const __nv_bfloat1
         }
         fence_before_sync();
     }
-    if (done) wait(bar_p, (done - 1) & 1u);
     if (done) {
+        wait(bar_p, (done - 1) & 1u);
+        add_p();
         atomicAdd(&s_db[(4 * ch4) & 31], dbs.x);
         atomicAdd(&s_db[(4 * ch4 + 1) & 31], dbs.y);
         atomicAdd(&s_db[(4 * ch4 + 2) & 31], dbs.z);
         atomicAdd(&s_db[(4 * ch4 + 3) & 31], dbs.w);
     }
-    __syncthreads();                                                       // every MMA of both contexts has completed
-    // ---- weight gradient of the CTA: P summed over its parts, then one addition per weight in global memory
-    float *acc = reinterpret_cast<float *>(gb + kOffCtx);                  // [kh * 3 + kw][ci][co]
-    for (int i = tid; i < 9 * 1024; i += kMidThreads) acc[i] = 0.f;
     __syncthreads();
-    if (done) {
-        const int m = (w8 & 3) * 32 + lane, h = (m >> 5) & 1, co = m & 31;
-#pragma unroll 1
-        for (int c = 0; c < 3; ++c) {
-            const int b = (w8 >> 2) * 3 + c, kw = b >> 1, r = b & 1;       // 32 columns: tap kw, grid row r
-            float v[32];
-            tmem_ld32_nowait(tmP + quarter + 32u * b, reinterpret_cast<uint32_t(&)[32]>(v));
-            tmem_wait_ld();
-            float *o = acc + (((r - h + 1) * 3 + kw) * 32) * 32 + co;
-#pragma unroll
-            for (int ci = 0; ci < 32; ++ci) atomicAdd(o + ci * 32, v[ci]);
-        }
-        fence_before_sync();
-    }
-    __syncthreads();
+    // ---- the CTA's weight gradient: one addition per weight in global memory
     for (int i = tid; i < 9 * 1024; i += kMidThreads) {
         const int co = i / 288, rem = i - co * 288, ci = rem / 9, kk = rem - ci * 9;
         atomicAdd(dW + i, acc[(kk * 32 + ci) * 32 + co]);

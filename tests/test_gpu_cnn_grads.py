@@ -115,3 +115,21 @@ def test_input_gradients_shrink_by_the_steps_of_the_largest_part():
         if where is not None:
             got = where.reshape(n, w, 2, 32).permute(0, 3, 2, 1).double()
             assert float((got - g).norm() / g.norm()) < 3.6e-7 * (3 - k), k
+
+
+@pytest.mark.parametrize("n,w", [(4096, 64), (1500, 300)])
+def test_weight_gradients_do_not_shrink_with_the_number_of_tiles(n, w):
+    """Layers 3 and 2: the projection on the 64-bit gradient, from which random rounding is absent. A tile's sum meets
+    8 steps of the largest part, layer 2's gradient also carries the shrinking of its input gradient (above)."""
+    c = inputs(n, w, 7)
+    grad, _, _ = backward(c)
+    P = layers(c["p"].double())
+    g = 2.0 * (c["y"].double() - c["target"].double()) / (4.0 * n * w)
+    for k, steps in ((3, None), (2, 8), (1, 12 + 8)):
+        a = c["acts"][k - 1].double()
+        if steps is not None:
+            ref = weight_grad(g, a, DIL[k]).reshape(-1)
+            got = grad[P[k][1]:P[k][2]].double()
+            shrink = float((got - ref) @ ref / (ref @ ref))
+            assert abs(shrink) < steps * 2.0 ** -25, (k, shrink)
+        g = input_grad(g, P[k][0], DIL[k]) * (a > 0)
