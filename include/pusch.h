@@ -475,6 +475,16 @@ pusch_status pusch_status_check(pusch_handle *h, const uint32_t *status, void *s
  */
 pusch_status pusch_selftest_wait(pusch_handle *h, unsigned limit_us, void *stream);
 
+/*
+ * The same check of the denoiser's kernels, which wait on their products: runs pusch_cnn_forward and
+ * pusch_cnn_backward (buffers as there) with every wait on a barrier that nothing completes, for limit_us
+ * microseconds (1 .. 1000000). After the first wait that expired a CTA goes on without waiting; its products in
+ * flight are waited for before it ends. The outputs are not valid.
+ */
+pusch_status pusch_selftest_cnn_wait(int n, int w, const void *x_bf16, const void *params_bf16, float *y, void *acts_bf16,
+                                     const float *target, float *grad, float *loss, float *work, unsigned limit_us,
+                                     void *stream);
+
 /* Message of the last non-OK status returned on this thread ("" if none). */
 const char *pusch_last_error(void);
 

@@ -43,7 +43,7 @@ EXPORTS = (
     "pusch_batch_create", "pusch_batch_destroy", "pusch_batch_sizes", "pusch_batch_run", "pusch_batch_autotune",
     "pusch_batch_tuning",
     "pusch_cnn_param_count", "pusch_cnn_forward", "pusch_cnn_backward", "pusch_cnn_adam", "pusch_ls_grid",
-    "pusch_chest_cnn", "pusch_status_check", "pusch_selftest_wait", "pusch_autotune",
+    "pusch_chest_cnn", "pusch_status_check", "pusch_selftest_wait", "pusch_selftest_cnn_wait", "pusch_autotune",
 )
 
 
@@ -134,6 +134,7 @@ def lib():
             "pusch_status_check": (I, [P, P, P]),
             "pusch_autotune": (I, [P, ctypes.c_char_p, P, ctypes.POINTER(I)]),
             "pusch_selftest_wait": (I, [P, ctypes.c_uint, P]),
+            "pusch_selftest_cnn_wait": (I, [I, I, P, P, P, P, P, P, P, P, ctypes.c_uint, P]),
             "pusch_last_error": (ctypes.c_char_p, []),
             "pusch_version": (ctypes.c_char_p, []),
         }
@@ -261,6 +262,12 @@ def pusch_autotune(h, cache_path=None, stream=None) -> int:
 
 def pusch_selftest_wait(h, limit_us: int, stream=None) -> None:
     _check(lib().pusch_selftest_wait(h, int(limit_us), _stream(stream)), "pusch_selftest_wait")
+
+
+def pusch_selftest_cnn_wait(n, w, x, params_bf16, y, acts, target, grad, loss, work, limit_us: int, stream=None) -> None:
+    _check(lib().pusch_selftest_cnn_wait(n, w, _ptr(x), _ptr(params_bf16), _ptr(y), _ptr(acts), _ptr(target), _ptr(grad),
+                                         _ptr(loss), _ptr(work), int(limit_us), _stream(stream)),
+           "pusch_selftest_cnn_wait")
 
 
 SLOT_STAGES = ("fft", "beamform", "ls", "detect")

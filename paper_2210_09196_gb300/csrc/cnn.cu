@@ -46,18 +46,19 @@ int cnn_param_count() { return param_offset(4); }
 // Forward pass of n grids of width w (cnn_tc.cu). x: [n][2][2][w] bf16, y: [n][2][2][w] f32; acts (or NULL):
 // [3][n][32][2][w] bf16, the post-ReLU activations.
 cudaError_t cnn_forward(int n, int w, const __nv_bfloat16 *x, const __nv_bfloat16 *P, float *y, __nv_bfloat16 *acts,
-                        cudaStream_t st, uint32_t *err) {
-    return launch_cnn_fwd(x, P, y, acts, n, w, err, st);
+                        cudaStream_t st, uint32_t *err, unsigned long long selftest_ns) {
+    return launch_cnn_fwd(x, P, y, acts, n, w, err, st, selftest_ns);
 }
 
 // Backward pass (cnn_bwd.cu): grad (zeroed here) = d mean((y - target)^2) / d params; *loss = that mean (if loss !=
 // NULL). work: 2 * n * 32 * 2 * w floats.
 cudaError_t cnn_backward(int n, int w, const __nv_bfloat16 *x, const __nv_bfloat16 *acts, const __nv_bfloat16 *P,
-                         const float *y, const float *target, float *grad, float *loss, float *work, cudaStream_t st) {
+                         const float *y, const float *target, float *grad, float *loss, float *work, cudaStream_t st,
+                         unsigned long long selftest_ns) {
     cudaError_t e;
     if ((e = cudaMemsetAsync(grad, 0, sizeof(float) * cnn_param_count(), st)) != cudaSuccess) return e;
     if (loss && (e = cudaMemsetAsync(loss, 0, sizeof(float), st)) != cudaSuccess) return e;
-    return launch_cnn_bwd(n, w, x, acts, P, y, target, grad, loss, work, nullptr, st);
+    return launch_cnn_bwd(n, w, x, acts, P, y, target, grad, loss, work, nullptr, st, selftest_ns);
 }
 
 cudaError_t cnn_adam(int step, float lr, float b1, float b2, float eps, float *p, __nv_bfloat16 *pb, const float *g,

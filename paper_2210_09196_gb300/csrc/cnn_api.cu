@@ -55,6 +55,27 @@ pusch_status pusch_cnn_backward(int n, int w, const void *x, const void *acts, c
     return PUSCH_OK;
 }
 
+pusch_status pusch_selftest_cnn_wait(int n, int w, const void *x, const void *params, float *y, void *acts,
+                                     const float *target, float *grad, float *loss, float *work, unsigned limit_us,
+                                     void *stream) {
+    pusch_status st = grid_check(n, w);
+    if (st != PUSCH_OK) return st;
+    if (limit_us < 1u || limit_us > 1000000u)
+        return cfail(PUSCH_ERR_ARG, "pusch_selftest_cnn_wait: limit_us out of [1, 1000000]");
+    if (n == 0) return PUSCH_OK;
+    if (!x || !params || !y || !acts || !target || !grad || !work)
+        return cfail(PUSCH_ERR_ARG, "pusch_selftest_cnn_wait: NULL buffer");
+    const __nv_bfloat16 *xb = (const __nv_bfloat16 *)x, *P = (const __nv_bfloat16 *)params;
+    cudaError_t e = pusch::cnn_forward(n, w, xb, P, y, (__nv_bfloat16 *)acts, (cudaStream_t)stream, nullptr,
+                                       1000ull * limit_us);
+    if (e == cudaSuccess)
+        e = pusch::cnn_backward(n, w, xb, (const __nv_bfloat16 *)acts, P, y, target, grad, loss, work,
+                                (cudaStream_t)stream, 1000ull * limit_us);
+    if (e != cudaSuccess) return cfail(PUSCH_ERR_CUDA, "CNN wait self-test launch", e);
+    pusch::set_last_error("");
+    return PUSCH_OK;
+}
+
 pusch_status pusch_cnn_adam(int step, float lr, float beta1, float beta2, float eps, float *params, void *params_bf16,
                             const float *grad, float *m, float *v, void *stream) {
     if (step < 1) return cfail(PUSCH_ERR_ARG, "Adam step counts from 1");

@@ -29,7 +29,9 @@
 // Measured (GB300, a step of 1024 grids x 256): out 41, mid 93 each, in 21 us; on FP32 FMAs (weights gradient: one thread
 // per channel pair) the backward pass took 4.0 ms. mid is bound by the chain load - split - products - mask of a tile,
 // of which two overlap (issue 23 %); out and in by the packed FMAs.
-// Every wait is bounded (2 s); after one that expired the threads go on without waiting and the error bit is set.
+// Every wait is bounded (2 s); after one that expired the threads go on without waiting, so that all barriers are met: no
+// address depends on what a wait was for. MMAs in flight are drained (bounded) before TMEM is freed, on a barrier of its
+// own: those of the products may be a phase behind by then.
 #include "tc_common.cuh"
 
 namespace pusch {
@@ -62,6 +64,7 @@ struct BwdArgs {
     int w, tiles, tiles_per_grid, dil;
     int vec;                 // the work buffer is 16-byte aligned
     float scale;             // 1 / count of the mean
+    unsigned long long selftest_ns;   // not 0: every wait is on a barrier that nothing completes, with this limit
 };
 
 constexpr int kTile = 128;
@@ -148,7 +151,7 @@ cnn_bwd_mid_kernel(BwdArgs g, const float *__restrict__ gout, const __nv_bfloat1
                    float *__restrict__ db, uint32_t *__restrict__ err) {
     chain_wait(gout, acts, W, gin, dW, db, err);
     extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(8) uint64_t bar_d[kCtx], bar_p[kCtx];
+    __shared__ __align__(8) uint64_t bar_d[kCtx], bar_p[kCtx], bar_drain[kCtx], bar_never;
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort, s_lock;
     __shared__ float s_db[32];
@@ -178,7 +181,9 @@ cnn_bwd_mid_kernel(BwdArgs g, const float *__restrict__ gout, const __nv_bfloat1
         for (int c = 0; c < kCtx; ++c) {
             mbar_init(smem_u32(&bar_d[c]), 1);
             mbar_init(smem_u32(&bar_p[c]), 1);
+            mbar_init(smem_u32(&bar_drain[c]), 1);
         }
+        mbar_init(smem_u32(&bar_never), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         s_abort = 0;
         s_lock = 0;
@@ -199,7 +204,12 @@ cnn_bwd_mid_kernel(BwdArgs g, const float *__restrict__ gout, const __nv_bfloat1
     const uint32_t tmD = s_tmem + (uint32_t)ctx * kCtxCols, tmP = tmD + 64u;
     const uint32_t quarter = (uint32_t)(w8 & 3) << 21;
     auto wait = [&](uint64_t *b, uint32_t ph) {
-        if (lane == 0) mbar_wait_sleep(smem_u32(&b[ctx]), ph, abort, err, 32);
+        if (lane == 0 && !*abort) {
+            if (g.selftest_ns)
+                mbar_wait_sleep(smem_u32(&bar_never), 0u, abort, err, 32, g.selftest_ns);
+            else
+                mbar_wait_sleep(smem_u32(&b[ctx]), ph, abort, err, 32);
+        }
         __syncwarp();
         fence_after_sync();
     };
@@ -362,8 +372,8 @@ cnn_bwd_mid_kernel(BwdArgs g, const float *__restrict__ gout, const __nv_bfloat1
     if (tid < 32) atomicAdd(db + tid, s_db[tid]);
     if (*abort) {                                                          // MMAs of a wait that expired
         if (w8 == 0 && elect_one()) {
-            mma_commit(smem_u32(&bar_d[ctx]));
-            mbar_drain(smem_u32(&bar_d[ctx]), done & 1u);
+            mma_commit(smem_u32(&bar_drain[ctx]));
+            mbar_drain(smem_u32(&bar_drain[ctx]), 0u);
         }
         __syncwarp();
     }
@@ -565,7 +575,7 @@ cnn_bwd_in_kernel(BwdArgs g, const float *__restrict__ gout, const __nv_bfloat16
 
 cudaError_t launch_cnn_bwd(int n, int w, const __nv_bfloat16 *x, const __nv_bfloat16 *acts, const __nv_bfloat16 *P,
                            const float *y, const float *target, float *grad, float *loss, float *work, uint32_t *err,
-                           cudaStream_t st) {
+                           cudaStream_t st, unsigned long long selftest_ns) {
     if (n == 0 || w == 0) return cudaSuccess;
     constexpr int kO2 = 32 * 2 * 9 + 32, kO3 = kO2 + 32 * 32 * 9 + 32, kO4 = kO3 + 32 * 32 * 9 + 32;
     const size_t big = (size_t)n * 64 * w;
@@ -577,6 +587,7 @@ cudaError_t launch_cnn_bwd(int n, int w, const __nv_bfloat16 *x, const __nv_bflo
     if (tiles > 0x3fffffffLL) return cudaErrorInvalidConfiguration;
     a.tiles = (int)tiles;
     a.dil = 0;
+    a.selftest_ns = selftest_ns;
     a.vec = reinterpret_cast<uintptr_t>(work) % 16 == 0;
     a.scale = 1.f / (float)((long long)n * 4 * w);
     cudaError_t e = cudaFuncSetAttribute(cnn_bwd_mid_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMidSmem);

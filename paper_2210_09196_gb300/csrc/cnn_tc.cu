@@ -28,7 +28,9 @@
 // HBM, with layers 1 and 4 on FP32 FMAs, the same took 780 us. Bound by the threads' share: per tile about 10 k clocks of
 // packed FMAs (layer 1), 5 k of bias, ReLU and packing, 6 k of waiting for products, four tiles overlapping.
 // Every wait is bounded (2 s); after one that expired the threads go on without waiting (the results are not valid and
-// the error bit says so), so all barriers are met; MMAs in flight are drained (bounded) before TMEM is freed.
+// the error bit says so), so all barriers are met: no address depends on what a wait was for. MMAs in flight are drained
+// (bounded) before TMEM is freed, on a barrier of its own: that of the products may be a phase behind by then, and a wait
+// for its newest phase would pass at once.
 #include "tc_common.cuh"
 
 namespace pusch {
@@ -52,6 +54,7 @@ static_assert(kOffW3 % 1024 == 0 && kOffW4 % 1024 == 0 && kOffCtx % 1024 == 0 &&
 struct FwdArgs {
     int w, in_ld, acts_ld, tiles, tiles_per_grid, step, halo;
     long long acts_layer;    // elements between two layers of acts
+    unsigned long long selftest_ns;   // not 0: every wait is on a barrier that nothing completes, with this limit
 };
 
 // Instruction descriptor of kind::f16 with BF16 A and B (format code 1), F32 accumulator, both K-major, M = 128.
@@ -72,7 +75,7 @@ cnn_fwd_kernel(FwdArgs g, const __nv_bfloat16 *__restrict__ in, const __nv_bfloa
                float *__restrict__ y, __nv_bfloat16 *__restrict__ acts, uint32_t *__restrict__ err) {
     chain_wait(in, P, y, acts, err);
     extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(8) uint64_t bars[kCtx];
+    __shared__ __align__(8) uint64_t bars[kCtx], bar_drain[kCtx], bar_never;
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
     __shared__ __align__(16) float s_bias[3][32];
@@ -123,7 +126,11 @@ cnn_fwd_kernel(FwdArgs g, const __nv_bfloat16 *__restrict__ in, const __nv_bfloa
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     if (tid == 0) {
-        for (int c = 0; c < kCtx; ++c) mbar_init(smem_u32(&bars[c]), 1);
+        for (int c = 0; c < kCtx; ++c) {
+            mbar_init(smem_u32(&bars[c]), 1);
+            mbar_init(smem_u32(&bar_drain[c]), 1);
+        }
+        mbar_init(smem_u32(&bar_never), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         s_abort = 0;
     }
@@ -153,7 +160,12 @@ cnn_fwd_kernel(FwdArgs g, const __nv_bfloat16 *__restrict__ in, const __nv_bfloa
         ctx_sync(ctx);
     };
     auto wait_products = [&]() {
-        if ((tid & 31) == 0) mbar_wait_sleep(bar, phase, abort, err, 32);
+        if ((tid & 31) == 0 && !*abort) {
+            if (g.selftest_ns)
+                mbar_wait_sleep(smem_u32(&bar_never), 0u, abort, err, 32, g.selftest_ns);
+            else
+                mbar_wait_sleep(bar, phase, abort, err, 32);
+        }
         __syncwarp();
         phase ^= 1u;
         fence_after_sync();
@@ -379,8 +391,8 @@ cnn_fwd_kernel(FwdArgs g, const __nv_bfloat16 *__restrict__ in, const __nv_bfloa
     // every MMA has completed: the last wait of each tile in flight covered them unless a wait expired
     if (*abort) {
         if (w4 == 0 && elect_one()) {
-            mma_commit(bar);
-            mbar_drain(bar, phase);
+            mma_commit(smem_u32(&bar_drain[ctx]));
+            mbar_drain(smem_u32(&bar_drain[ctx]), 0u);
         }
         __syncwarp();
     }
@@ -395,9 +407,10 @@ cnn_fwd_kernel(FwdArgs g, const __nv_bfloat16 *__restrict__ in, const __nv_bfloa
 }  // namespace
 
 cudaError_t launch_cnn_fwd(const __nv_bfloat16 *in, const __nv_bfloat16 *P, float *y, __nv_bfloat16 *acts, int n, int w,
-                           uint32_t *err, cudaStream_t st) {
+                           uint32_t *err, cudaStream_t st, unsigned long long selftest_ns) {
     if (n == 0 || w == 0) return cudaSuccess;
     FwdArgs a;
+    a.selftest_ns = selftest_ns;
     a.w = w;
     a.in_ld = w;
     a.acts_ld = w;

@@ -252,16 +252,18 @@ inline cudaError_t launch_beamform(const Geometry &g, int n_slots, const void *f
 
 // Learned channel-estimate denoiser (cnn.cu). Parameters packed per layer as W[co][ci][3][3], b[co].
 int cnn_param_count();
-// acts may be NULL; err (optional): error word of the kernel's bounded waits.
+// acts may be NULL; err (optional): error word of the kernel's bounded waits; selftest_ns: not 0 makes every wait expire
+// after that long.
 cudaError_t cnn_forward(int n, int w, const __nv_bfloat16 *x, const __nv_bfloat16 *P, float *y, __nv_bfloat16 *acts,
-                        cudaStream_t st, uint32_t *err = nullptr);
+                        cudaStream_t st, uint32_t *err = nullptr, unsigned long long selftest_ns = 0);
 cudaError_t launch_cnn_fwd(const __nv_bfloat16 *in, const __nv_bfloat16 *P, float *y, __nv_bfloat16 *acts, int n, int w,
-                           uint32_t *err, cudaStream_t st);
+                           uint32_t *err, cudaStream_t st, unsigned long long selftest_ns);
 cudaError_t cnn_backward(int n, int w, const __nv_bfloat16 *x, const __nv_bfloat16 *acts, const __nv_bfloat16 *P,
-                         const float *y, const float *target, float *grad, float *loss, float *work, cudaStream_t st);
+                         const float *y, const float *target, float *grad, float *loss, float *work, cudaStream_t st,
+                         unsigned long long selftest_ns = 0);
 cudaError_t launch_cnn_bwd(int n, int w, const __nv_bfloat16 *x, const __nv_bfloat16 *acts, const __nv_bfloat16 *P,
                            const float *y, const float *target, float *grad, float *loss, float *work, uint32_t *err,
-                           cudaStream_t st);
+                           cudaStream_t st, unsigned long long selftest_ns);
 cudaError_t cnn_adam(int step, float lr, float b1, float b2, float eps, float *p, __nv_bfloat16 *pb, const float *g,
                      float *m, float *v, cudaStream_t st);
 cudaError_t launch_ls_grid(const Geometry &g, int n_slots, const float2 *beam, const float2 *pilots,

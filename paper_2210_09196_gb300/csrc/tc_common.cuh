@@ -65,12 +65,12 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 // mbar_wait with a pause of about `sleep_ns` between polls, for waits that usually last a while (another role's
 // work): the polling lane then leaves the issue slots to the warps that do that work.
 __device__ __forceinline__ bool mbar_wait_sleep(uint32_t bar, uint32_t parity, volatile int *abort, uint32_t *err,
-                                                unsigned sleep_ns) {
+                                                unsigned sleep_ns, uint64_t limit_ns = kWaitNs) {
     for (int k = 0; k < kPollsPerTimer; ++k) {
         if (mbar_try_wait(bar, parity)) return true;
         __nanosleep(sleep_ns);
     }
-    const uint64_t deadline = globaltimer() + kWaitNs;
+    const uint64_t deadline = globaltimer() + limit_ns;
     for (;;) {
         for (int k = 0; k < kPollsPerTimer; ++k) {
             if (mbar_try_wait(bar, parity)) return true;
