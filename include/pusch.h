@@ -77,7 +77,9 @@ typedef enum {
  * Every kernel that waits on asynchronous copies or MMAs gives up after 2 s and sets a bit in an error word
  * of its handle (or batch, or no-alloc call) instead of hanging; pusch_slot, pusch_slot_host,
  * pusch_mmse_detect, pusch_batch_run and pusch_slot_noalloc move that word into status[0] / status[3] at
- * their end (pusch_mmse_detect also reports expiries of the handle's earlier stage calls) and clear it. */
+ * their end (pusch_mmse_detect also reports expiries of the handle's earlier stage calls) and clear it.
+ * pusch_cnn_forward and pusch_cnn_backward have no handle: what they could not finish comes out as NaN, in the
+ * loss too. */
 #define PUSCH_STATUS_PIVOT 0x1u     /* Cholesky met a non-positive or non-finite pivot            */
 #define PUSCH_STATUS_NONFINITE 0x2u /* a detected symbol came out non-finite                      */
 #define PUSCH_STATUS_TIMEOUT 0x4u   /* a bounded device wait expired: the call's outputs are not valid */
@@ -476,10 +478,11 @@ pusch_status pusch_status_check(pusch_handle *h, const uint32_t *status, void *s
 pusch_status pusch_selftest_wait(pusch_handle *h, unsigned limit_us, void *stream);
 
 /*
- * The same check of the denoiser's kernels, which wait on their products: runs pusch_cnn_forward and
- * pusch_cnn_backward (buffers as there) with every wait on a barrier that nothing completes, for limit_us
- * microseconds (1 .. 1000000). After the first wait that expired a CTA goes on without waiting; its products in
- * flight are waited for before it ends. The outputs are not valid.
+ * The same check of the denoiser's kernels, which wait on their products: runs pusch_cnn_backward on the given y
+ * and acts, then pusch_cnn_forward (buffers as there), with every wait on a barrier that nothing completes, for
+ * limit_us microseconds (1 .. 1000000). After the first wait that expired a CTA goes on without waiting; its
+ * products in flight are waited for before it ends. What they lead to comes out as NaN: the loss and the gradients
+ * of the first three layers (the last layer's kernel waits for nothing), then y.
  */
 pusch_status pusch_selftest_cnn_wait(int n, int w, const void *x_bf16, const void *params_bf16, float *y, void *acts_bf16,
                                      const float *target, float *grad, float *loss, float *work, unsigned limit_us,

@@ -66,11 +66,10 @@ pusch_status pusch_selftest_cnn_wait(int n, int w, const void *x, const void *pa
     if (!x || !params || !y || !acts || !target || !grad || !work)
         return cfail(PUSCH_ERR_ARG, "pusch_selftest_cnn_wait: NULL buffer");
     const __nv_bfloat16 *xb = (const __nv_bfloat16 *)x, *P = (const __nv_bfloat16 *)params;
-    cudaError_t e = pusch::cnn_forward(n, w, xb, P, y, (__nv_bfloat16 *)acts, (cudaStream_t)stream, nullptr,
-                                       1000ull * limit_us);
+    cudaError_t e = pusch::cnn_backward(n, w, xb, (const __nv_bfloat16 *)acts, P, y, target, grad, loss, work,
+                                        (cudaStream_t)stream, 1000ull * limit_us);
     if (e == cudaSuccess)
-        e = pusch::cnn_backward(n, w, xb, (const __nv_bfloat16 *)acts, P, y, target, grad, loss, work,
-                                (cudaStream_t)stream, 1000ull * limit_us);
+        e = pusch::cnn_forward(n, w, xb, P, y, (__nv_bfloat16 *)acts, (cudaStream_t)stream, nullptr, 1000ull * limit_us);
     if (e != cudaSuccess) return cfail(PUSCH_ERR_CUDA, "CNN wait self-test launch", e);
     pusch::set_last_error("");
     return PUSCH_OK;

@@ -29,7 +29,8 @@
 // Measured (GB300, a step of 1024 grids x 256): out 41, mid 93 each, in 21 us; on FP32 FMAs (weights gradient: one thread
 // per channel pair) the backward pass took 4.0 ms. mid is bound by the chain load - split - products - mask of a tile,
 // of which two overlap (issue 23 %); out and in by the packed FMAs.
-// Every wait is bounded (2 s); after one that expired the threads go on without waiting, so that all barriers are met: no
+// Every wait is bounded (2 s); after one that expired the loss and the CTA's gradients are NaN, which the layers before take
+// over, the error bit, where there is an error word, is set, and the threads go on without waiting, so all barriers are met: no
 // address depends on what a wait was for. MMAs in flight are drained (bounded) before TMEM is freed, on a barrier of its
 // own: those of the products may be a phase behind by then.
 #include "tc_common.cuh"
@@ -68,6 +69,7 @@ struct BwdArgs {
 };
 
 constexpr int kTile = 128;
+__device__ __forceinline__ float nan_value() { return __int_as_float(0x7fffffff); }
 
 // the gradients' rows in the work buffer, which may be aligned to its floats only
 __device__ __forceinline__ float4 load4(const float *p, int vec) {
@@ -148,8 +150,8 @@ __device__ __forceinline__ void lock_release(int *lock) {
 __global__ void __launch_bounds__(kMidThreads, 1)
 cnn_bwd_mid_kernel(BwdArgs g, const float *__restrict__ gout, const __nv_bfloat16 *__restrict__ acts,
                    const __nv_bfloat16 *__restrict__ W, float *__restrict__ gin, float *__restrict__ dW,
-                   float *__restrict__ db, uint32_t *__restrict__ err) {
-    chain_wait(gout, acts, W, gin, dW, db, err);
+                   float *__restrict__ db, float *__restrict__ loss, uint32_t *__restrict__ err) {
+    chain_wait(gout, acts, W, gin, dW, db, loss, err);
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t bar_d[kCtx], bar_p[kCtx], bar_drain[kCtx], bar_never;
     __shared__ uint32_t s_tmem;
@@ -337,6 +339,7 @@ cnn_bwd_mid_kernel(BwdArgs g, const float *__restrict__ gout, const __nv_bfloat1
             tmem_ld32_nowait(tmD + quarter + 32u * half, reinterpret_cast<uint32_t(&)[32]>(v));
             tmem_wait_ld();
             float *o = gin + ((long long)gi * g.w + x) * 64 + half * 32;
+            const bool lost = *abort;                                      // a wait of this CTA expired
             if (x < g.w) {
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
@@ -345,8 +348,8 @@ cnn_bwd_mid_kernel(BwdArgs g, const float *__restrict__ gout, const __nv_bfloat1
                     float r[8];
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
-                        r[2 * e] = __uint_as_float(u[e] << 16) > 0.f ? v[8 * c + 2 * e] : 0.f;
-                        r[2 * e + 1] = __uint_as_float(u[e] & 0xffff0000u) > 0.f ? v[8 * c + 2 * e + 1] : 0.f;
+                        r[2 * e] = lost ? nan_value() : __uint_as_float(u[e] << 16) > 0.f ? v[8 * c + 2 * e] : 0.f;
+                        r[2 * e + 1] = lost ? nan_value() : __uint_as_float(u[e] & 0xffff0000u) > 0.f ? v[8 * c + 2 * e + 1] : 0.f;
                     }
                     store4(o + 8 * c, r[0], r[1], r[2], r[3], g.vec);
                     store4(o + 8 * c + 4, r[4], r[5], r[6], r[7], g.vec);
@@ -367,9 +370,10 @@ cnn_bwd_mid_kernel(BwdArgs g, const float *__restrict__ gout, const __nv_bfloat1
     // ---- the CTA's weight gradient: one addition per weight in global memory
     for (int i = tid; i < 9 * 1024; i += kMidThreads) {
         const int co = i / 288, rem = i - co * 288, ci = rem / 9, kk = rem - ci * 9;
-        atomicAdd(dW + i, acc[(kk * 32 + ci) * 32 + co]);
+        atomicAdd(dW + i, *abort ? nan_value() : acc[(kk * 32 + ci) * 32 + co]);
     }
-    if (tid < 32) atomicAdd(db + tid, s_db[tid]);
+    if (tid < 32) atomicAdd(db + tid, *abort ? nan_value() : s_db[tid]);
+    if (tid == 0 && loss && *abort) atomicAdd(loss, nan_value());
     if (*abort) {                                                          // MMAs of a wait that expired
         if (w8 == 0 && elect_one()) {
             mma_commit(smem_u32(&bar_drain[ctx]));
@@ -602,11 +606,11 @@ cudaError_t launch_cnn_bwd(int n, int w, const __nv_bfloat16 *x, const __nv_bflo
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     a.dil = 16;
     launch_chained(true, cnn_bwd_mid_kernel, dim3(one), dim3(kMidThreads), kMidSmem, st, a, gbuf, acts + big, P + kO3, ga, grad + kO3,
-                                                           grad + kO3 + 32 * 32 * 9, err);
+                                                           grad + kO3 + 32 * 32 * 9, loss, err);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     a.dil = 8;
     launch_chained(true, cnn_bwd_mid_kernel, dim3(one), dim3(kMidThreads), kMidSmem, st, a, ga, acts, P + kO2, gbuf, grad + kO2,
-                                                           grad + kO2 + 32 * 32 * 9, err);
+                                                           grad + kO2 + 32 * 32 * 9, loss, err);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     launch_chained(true, cnn_bwd_in_kernel, dim3(three), dim3(kEndThreads), 0, st, a, gbuf, x, grad, grad + 32 * 2 * 9);
     return cudaGetLastError();

@@ -27,8 +27,8 @@
 // Measured (GB300, 512 grids of 3276 subcarriers): 190 us, 460 TFLOP/s of the network's arithmetic; layer by layer through
 // HBM, with layers 1 and 4 on FP32 FMAs, the same took 780 us. Bound by the threads' share: per tile about 10 k clocks of
 // packed FMAs (layer 1), 5 k of bias, ReLU and packing, 6 k of waiting for products, four tiles overlapping.
-// Every wait is bounded (2 s); after one that expired the threads go on without waiting (the results are not valid and
-// the error bit says so), so all barriers are met: no address depends on what a wait was for. MMAs in flight are drained
+// Every wait is bounded (2 s); after one that expired the threads go on without waiting (the CTA's outputs from then on are
+// NaN and the error bit, where the caller has an error word, is set), so all barriers are met: no address depends on what a wait was for. MMAs in flight are drained
 // (bounded) before TMEM is freed, on a barrier of its own: that of the products may be a phase behind by then, and a wait
 // for its newest phase would pass at once.
 #include "tc_common.cuh"
@@ -375,6 +375,7 @@ cnn_fwd_kernel(FwdArgs g, const __nv_bfloat16 *__restrict__ in, const __nv_bfloa
             if (!mine[b]) continue;
             const int i = row + 128 * b;
             float *o = y + (long long)gi * 4 * g.w + x + 128 * b;
+            const bool lost = *abort;                                       // a wait of this CTA expired
 #pragma unroll
             for (int co = 0; co < 2; ++co)
 #pragma unroll
@@ -382,7 +383,7 @@ cnn_fwd_kernel(FwdArgs g, const __nv_bfloat16 *__restrict__ in, const __nv_bfloa
                     float v = s_bias4[co] + sums[i * 13 + 4 + h * 2 + co];
                     if (i > 0) v += sums[(i - 1) * 13 + h * 2 + co];
                     if (i < kRows - 1) v += sums[(i + 1) * 13 + 8 + h * 2 + co];
-                    o[(long long)(co * 2 + h) * g.w] = v + res[b][co * 2 + h];
+                    o[(long long)(co * 2 + h) * g.w] = lost ? __int_as_float(0x7fffffff) : v + res[b][co * 2 + h];
                 }
         }
         // (the next tile's first barrier orders these reads before the activations are written again)

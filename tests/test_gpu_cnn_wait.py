@@ -58,3 +58,16 @@ def test_selftest_arguments():
             B.pusch_selftest_cnn_wait(1, 8, b["x"], b["p"], b["y"], b["acts"], b["target"], b["grad"], b["loss"],
                                       b["work"], limit)
         assert ei.value.code == B.PUSCH_ERR_ARG
+
+
+@pytest.mark.parametrize("n,w", [(1, 40), (2000, 130)])
+def test_expired_waits_show_in_the_outputs(n, w):
+    """The backward pass runs on valid forward results, so what is not finite in its outputs it made so itself."""
+    b = buffers(n, w)
+    step(b, n, w)
+    selftest(b, n, w)
+    torch.cuda.synchronize()
+    last = 2 * 32 * 9 + 2                                  # layer 4's gradients come from a kernel without waits
+    assert bool(b["loss"].isnan().all()) and bool(b["grad"][:-last].isnan().all())
+    assert not bool(b["grad"][-last:].isnan().any())
+    assert bool(b["y"].isnan().all())
