@@ -528,14 +528,18 @@ Tf32Plan tf32_plan(const Geometry &g) {
 
 }  // namespace
 
-// The kernel's time hardly depends on the beams (it is bound by its loading), that of the FP32 kernel goes with them
-// in steps of 8, 16, 32 and 64. Measured at 64 antennas, 8 slots of 3275 subcarriers: 8 beams 134 us against 111 us
-// on FP32 FMAs, 24 beams 146 against 201; at 48 antennas and 31 beams 139 against 207. With up to 32 beams and less
-// than two tiles per SM the FP32 kernel's smaller tiles win (64 x 24 x 333, one slot: 11 us against 15).
-bool bf_tf32k_supported(const Geometry &g, int n_slots) {
+// By the geometry alone, never by the number of slots: a slot's values must not depend on the batch that it is in (the
+// two kernels round differently). The kernel's time hardly depends on the beams (it is bound by its loading), that of the
+// FP32 kernel goes with them in steps of 8, 16, 32 and 64. FP32 FMAs against this kernel, us, one slot / 12 slots:
+//   more than 32 beams       32 x 33 x 101: 11 / 10;  64 x 40 x 25: 15 / 13;  256 x 64 x 333: 83 / 25 (one slot)
+//   more than 64 antennas    72 x 24 x 129: 15, 35 / 12, 31;  96 x 32 x 257: 15, 48 / 14, 47;  96 x 32 x 1153: 23, 164 / 20, 131
+//   33..64 antennas          64 x 24: 385 subcarriers 11, 52 / 13, 42;  513: 11, 59 / 13, 48;  641: 16, 70 / 13, 55
+//   32 antennas              32 x 24: 641 subcarriers 10, 39 / 11, 35;  1025: 11, 56 / 11, 47;  2305: 15, 117 / 14, 92
+// so at 17..32 beams and up to 64 antennas the line lies where one slot is about even. At 8 beams the FP32 kernel is
+// faster (64 antennas, 3275 subcarriers, 8 slots: 111 against 134 us).
+bool bf_tf32k_supported(const Geometry &g) {
     if (g.form != PUSCH_FORM_FP32 || !tf32_plan(g).ok || g.n_rx < 32 || g.n_beams <= 16) return false;
-    const long long tiles = (long long)n_slots * g.n_sym * ((g.n_sc + kTileM - 1) / kTileM);
-    return g.n_beams > 32 || tiles >= 2 * 152;
+    return g.n_beams > 32 || g.n_rx > 64 || g.n_sc > (g.n_rx > 32 ? 512 : 1024);
 }
 
 cudaError_t launch_beamform_tf32k(const Geometry &g, int n_slots, const float2 *freq, const float2 *W, float2 *beam,

@@ -230,7 +230,7 @@ cudaError_t launch_beamform_tf32(const Geometry &g, int n_slots, const float2 *f
                                  uint32_t *err_word, cudaStream_t st);
 // The same product with the antennas split over a cluster of CTAs (beamform_tf32k.cu): up to 256 antennas, any
 // subcarrier count, beam count and alignment; true where it is faster than the FP32 FMAs.
-bool bf_tf32k_supported(const Geometry &g, int n_slots);
+bool bf_tf32k_supported(const Geometry &g);
 cudaError_t launch_beamform_tf32k(const Geometry &g, int n_slots, const float2 *freq, const float2 *W, float2 *beam,
                                   uint32_t *err_word, cudaStream_t st);
 // Beamforming of the FFT output in the geometry's form (FP32: 3xTF32 tensor cores, with the whole of W per CTA where
@@ -245,7 +245,7 @@ inline cudaError_t launch_beamform(const Geometry &g, int n_slots, const void *f
                                    fp8_scales(g, n_slots, const_cast<void *>(freq)), W, beam, err_word, st, tune);
     if (bf_tf32_supported(g) && reinterpret_cast<uintptr_t>(freq) % 16 == 0 && reinterpret_cast<uintptr_t>(beam) % 16 == 0)
         return launch_beamform_tf32(g, n_slots, static_cast<const float2 *>(freq), W, beam, err_word, st);
-    if (bf_tf32k_supported(g, n_slots))
+    if (bf_tf32k_supported(g))
         return launch_beamform_tf32k(g, n_slots, static_cast<const float2 *>(freq), W, beam, err_word, st);
     return launch_beamform_fp32(g, n_slots, static_cast<const float2 *>(freq), W, beam, st);
 }
