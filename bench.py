@@ -219,8 +219,11 @@ def kernel_of(stage, form, cell=None):
     if stage == "beamform" and form == "fp32" and cell is not None and not (
             cell.n_sc % 2 == 0 and cell.n_rx % 16 == 0 and cell.n_beams % 8 == 0 and cell.n_beams <= 64
             and 32 * cell.n_rx * cell.n_beams <= 96 * 1024):
-        # the whole of W does not fit one CTA: the antennas are split over a cluster, or FP32 FMAs
-        return k["fp32_k" if 32 <= cell.n_rx <= 256 and cell.n_beams > 32 else "fp32_simt"]
+        # not the kernel that keeps the whole of W in one CTA: the antennas split over a cluster, or FP32 FMAs (the rule
+        # of bf_tf32k_supported)
+        split = 32 <= cell.n_rx <= 256 and 16 < cell.n_beams <= 64 and (
+            cell.n_beams > 32 or cell.n_rx > 64 or cell.n_sc > (512 if cell.n_rx > 32 else 1024))
+        return k["fp32_k" if split else "fp32_simt"]
     return k[form] if isinstance(k, dict) else k
 
 
