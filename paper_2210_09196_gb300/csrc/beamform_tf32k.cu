@@ -568,29 +568,17 @@ cudaError_t launch_beamform_tf32k(const Geometry &g, int n_slots, const float2 *
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaLaunchConfig_t cfg{};
-    cudaLaunchAttribute at[2];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)p.cluster;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = p.smem;
-    cfg.stream = st;
-    cfg.attrs = at;
-    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // launch_chained, with a cluster
-    at[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.numAttrs = 2;
+    ChainedConfig c(g.chained, dim3((unsigned)(sms / p.cluster * p.cluster)), dim3(kThreads), p.smem, st,
+                    (unsigned)p.cluster);
     // as many clusters as are resident at once (36 of 4 CTAs on 152 SMs): the tiles are dealt out evenly, so a
     // cluster that had to wait for a place would double the time
     int clusters = sms;
-    cfg.gridDim = dim3((unsigned)(sms / p.cluster * p.cluster));
-    if (p.cluster > 1 && (e = cudaOccupancyMaxActiveClusters(&clusters, beamform_tf32k_kernel, &cfg)) != cudaSuccess)
+    if (p.cluster > 1 && (e = cudaOccupancyMaxActiveClusters(&clusters, beamform_tf32k_kernel, &c.cfg)) != cudaSuccess)
         return e;
     if (clusters < 1) return cudaErrorInvalidConfiguration;
     if (clusters > tiles) clusters = (int)tiles;
-    cfg.gridDim = dim3((unsigned)(clusters * p.cluster));
-    if ((e = cudaLaunchKernelEx(&cfg, beamform_tf32k_kernel, a, freq, W, beam, err_word)) != cudaSuccess) return e;
+    c.cfg.gridDim = dim3((unsigned)(clusters * p.cluster));
+    if ((e = cudaLaunchKernelEx(&c.cfg, beamform_tf32k_kernel, a, freq, W, beam, err_word)) != cudaSuccess) return e;
     return cudaGetLastError();
 }
 

@@ -61,21 +61,31 @@ __device__ __forceinline__ void chain_wait(T &...p) {
 }
 // Lets the next kernel of the chain start (all CTAs have to have called it or ended).
 __device__ __forceinline__ void chain_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-// chained = false: an ordinary launch (the waits inside pass at once).
+// chained = false: an ordinary launch (the waits inside pass at once). cluster: CTAs per thread-block cluster.
+struct ChainedConfig {
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at[2];
+    ChainedConfig(bool chained, dim3 grid, dim3 block, size_t smem, cudaStream_t st, unsigned cluster = 1) {
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = chained ? 1 : 0;
+        at[1].id = cudaLaunchAttributeClusterDimension;
+        at[1].val.clusterDim.x = cluster;
+        at[1].val.clusterDim.y = 1;
+        at[1].val.clusterDim.z = 1;
+        cfg.gridDim = grid;
+        cfg.blockDim = block;
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = st;
+        cfg.attrs = at;
+        cfg.numAttrs = cluster > 1 ? 2 : 1;
+    }
+    ChainedConfig(const ChainedConfig &) = delete;
+};
 template <typename... P, typename... A>
 inline cudaError_t launch_chained(bool chained, void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                                   A... args) {
-    cudaLaunchConfig_t cfg{};
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = chained ? 1 : 0;
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
+    const ChainedConfig c(chained, grid, block, smem, st);
+    return cudaLaunchKernelEx(&c.cfg, k, static_cast<P>(args)...);
 }
 
 // ---------------------------------------------------------------------------------- derived geometry
