@@ -50,7 +50,10 @@ typedef enum {
 
 /* Arithmetic form of the chain. */
 typedef enum {
-    PUSCH_FORM_FP32 = 0,   /* plain: FFT and beamforming in FP32, intermediates stored as c64           */
+    PUSCH_FORM_FP32 = 0,   /* plain: FFT and beamforming to FP32 accuracy, intermediates stored as c64. The
+                              larger beamforming shapes run on the tensor cores from TF32 operands split in
+                              two parts (three products each, FP32 accumulation); they hold FP32 accuracy
+                              for samples from 2^-114 (5e-35) up.                                        */
     PUSCH_FORM_MIXED = 1,  /* FFT output stored as FP16 (4096-point rows of FP16 samples on the tcgen05
                               tensor cores with FP16 operands and FP32 accumulation, other shapes in FP32
                               registers); beamforming on the tensor cores with FP16 operands and FP32

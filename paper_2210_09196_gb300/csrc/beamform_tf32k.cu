@@ -6,7 +6,7 @@
 // Im W[r][b], B[2b + 1][2r] = -Im W[r][b], B[2b + 1][2r + 1] = Re W[r][b]. Every FP32 operand v is split
 // into two TF32 values, hi = TF32(v) and lo = TF32(v - hi), so that hi + lo holds v to
 // about 2^-23, and D = A_hi B_hi + (A_hi B_lo + A_lo B_hi) (the dropped A_lo B_lo is below 2^-22 of |A||B|).
-// Inputs that are not finite give results that are not finite.
+// Infinities and NaN give what they give in FP32 arithmetic.
 //
 // B (hi and lo) stays in shared memory, 16 bytes per (beam row, antenna): 128 KB hold 64 antennas at 64 beams.
 // So a cluster of 1, 2 or 4 CTAs shares one 128-subcarrier tile, each CTA forming the product over its own
@@ -33,7 +33,7 @@
 // 16 warps leave 128 registers a thread: with more, the 64 columns of E that an epilogue thread holds spilled, and
 // the spills, missing the little L1 beside 227 KB of shared memory, took 12 k clocks per tile.
 //
-// Measured (GB300, 2 slots of 256 antennas, 64 beams, 3276 subcarriers): 163 us against 671 us on FP32 FMAs; bound by
+// Measured (GB300, 2 slots of 256 antennas, 64 beams, 3276 subcarriers): 166 us against 671 us on FP32 FMAs; bound by
 // the instructions of the warps that load and split (about 900 clocks per stage; HBM needs 440).
 //
 // Every wait is bounded (%globaltimer, 2 s); on expiry the CTA records a timeout in err_word bit 0, all roles
@@ -76,9 +76,15 @@ struct Tf32Shared {
 };
 
 // v = hi + lo in TF32: hi rounded to nearest (ties away from zero), lo the exact remainder, of which the tensor core
-// reads the upper 11 bits of at most 12 (below 2^-23 of |v| is lost).
+// reads the upper 11 bits of at most 12 (below 2^-23 of |v| is lost; below |v| = 2^-114, where lo leaves the normal
+// range, more). hi stays finite: it is rounded from v brought to the largest magnitude that does not round to infinity,
+// so that values next to FLT_MAX keep theirs in lo, and an infinity or a NaN is in lo alone and gives what it gives in
+// FP32 arithmetic (as hi an infinity would meet both parts of the other operand, whose signs may differ, and its lo were
+// a NaN). The limit is one instruction of some eight per value: 162.5 -> 165.7 us for the case above.
 __device__ __forceinline__ void split_tf32(float x, uint32_t &hi, uint32_t &lo) {
-    hi = (__float_as_uint(x) + 0x1000u) & 0xffffe000u;
+    float c;   // x with its magnitude limited
+    asm("min.xorsign.abs.f32 %0, %1, %2;" : "=f"(c) : "f"(x), "f"(__uint_as_float(0x7f7fefffu)));
+    hi = (__float_as_uint(c) + 0x1000u) & 0xffffe000u;
     lo = __float_as_uint(x - __uint_as_float(hi));
 }
 
