@@ -302,6 +302,9 @@ pusch_status pusch_destroy(pusch_handle *h) {
     cudaFree(h->h_xhat);
     cudaFree(h->h_bits);
     cudaFree(h->h_status);
+    cudaFree(h->cnn_grid);
+    cudaFree(h->cnn_scale);
+    cudaFree(h->cnn_y);
     delete h;
     return ok();
 }
