@@ -21,9 +21,12 @@
 //     kappa of one k0 go to stage 2's operand as one 8-byte store. The padded strides of that operand (144 B
 //     between core matrices along K, 1184 B between groups of eight columns) spread the stores over the banks.
 //   - Stage 2's columns are ordered so that a lane's eight column groups are eight consecutive output positions
-//     on a 16-byte boundary of the plane and the four lanes of a row 64 consecutive bytes: position (bin + n_sc / 2)
-//     mod 4096, octet e = t + 4 half. The FFT shift's remainder hr = (n_sc / 2) mod 8 rotates k0; only octet 0 then
-//     mixes two k1, and its first hr elements come from the lanes of k1 - 1 (eight exchanges per 64 x 8 block).
+//     on a 16-byte boundary in memory and the four lanes of a row 64 consecutive bytes: position (bin + n_sc / 2)
+//     mod 4096, octet e = t + 4 half. The remainder hr = (n_sc / 2 + off) mod 8, off the output's distance from a
+//     16-byte boundary in values, rotates k0; only octet 0 then mixes two k1, and its first hr elements come from the
+//     lanes of k1 - 1 (eight exchanges per 64 x 8 block). Where off > 0, the octets over a plane's ends are stored
+//     value by value (7,168 rows into a plane 2, 4 or 8 bytes off a boundary: 187, 194 and 205 us when all values were
+//     stored singly, aligned 59.6).
 // A 4096-point transform thus costs two MMA passes (8 MMAs of 128 x 128 x 16) and one pass of twiddles and
 // transposition through shared memory.
 //
@@ -122,9 +125,11 @@ __device__ __forceinline__ uint32_t pack_half2(float a, float b) {
 struct FftTcArgs {
     long long rows;
     int n_sc, pitch;
-    int vec;     // the output is 16-byte aligned
+    int off;     // values from the last 16-byte boundary to the output
 };
 
+// OFF: the output is not on a 16-byte boundary (compiled apart: the stores over the planes' ends cost the aligned case 2 %)
+template <bool OFF>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 fft_tc_kernel(const __grid_constant__ CUtensorMap tin, __half *__restrict__ out, const float2 *__restrict__ tw,
               FftTcArgs g, uint32_t *__restrict__ err) {
@@ -266,13 +271,13 @@ fft_tc_kernel(const __grid_constant__ CUtensorMap tin, __half *__restrict__ out,
         float2 pw[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i) pw[i] = __ldg(&tw[(4 * i + t) * g8]);
-        const int h = g.n_sc >> 1, hr = h & 7, hb = h - hr;
+        const int h = g.n_sc >> 1, hr = (h + (OFF ? g.off : 0)) & 7, hb = h - hr;   // hb + off: a multiple of 8
         uint32_t first[4];   // the halves of octet 0's pairs that lie among its first hr elements
 #pragma unroll
         for (int i = 0; i < 4; ++i) first[i] = t > 0 ? 0u : hr - 2 * i >= 2 ? 0xffffffffu : hr - 2 * i == 1 ? 0xffffu : 0u;
         // this lane's element of the warp's two edge octets: lane = [edge][plane][element]; -1: none
-        const int ei = lane & 7, epos = ((64 * 16 * (warp + (lane >> 4)) + hb) & (kN - 1)) + ei;
-        const bool emine = g.vec && hr > 0 && (lane < 16 ? ei >= hr : ei < hr) && epos < g.pitch;
+        const int ei = lane & 7, epos = (64 * 16 * (warp + (lane >> 4)) + hb + ei) & (kN - 1);
+        const bool emine = hr > 0 && (lane < 16 ? ei >= hr : ei < hr) && epos < g.pitch;
         const int eout = emine ? epos + ((lane >> 3) & 1) * g.pitch : -1;
         uint32_t acc_phase = 0;
         for (long long it = 0; it < n_my; ++it) {
@@ -334,17 +339,6 @@ fft_tc_kernel(const __grid_constant__ CUtensorMap tin, __half *__restrict__ out,
                 }
                 // element i of the octet goes to position a0 + i; of octet 0 the first hr one block further on
                 const int a0 = (8 * e + 64 * k1 + hb) & (kN - 1);
-                if (!g.vec) {
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const int a = (a0 + i + (e == 0 && i < hr ? 64 : 0)) & (kN - 1), sh = 16 * (i & 1);
-                        if (a < g.pitch) {
-                            o[a] = __ushort_as_half((unsigned short)(a < g.n_sc ? v[i >> 1] >> sh : 0u));
-                            o[g.pitch + a] = __ushort_as_half((unsigned short)(a < g.n_sc ? v[4 + (i >> 1)] >> sh : 0u));
-                        }
-                    }
-                    continue;
-                }
                 if (half == 0 && hr > 0) {
                     uint32_t rot[8];
 #pragma unroll
@@ -362,7 +356,7 @@ fft_tc_kernel(const __grid_constant__ CUtensorMap tin, __half *__restrict__ out,
                     }
                 }
                 const bool whole = !(c == 0 && lane == 0 && hr > 0);
-                if (whole && a0 < g.pitch) {
+                if (whole && (OFF ? a0 + 8 <= g.pitch : a0 < g.pitch)) {
                     if (a0 + 8 > g.n_sc) {
 #pragma unroll
                         for (int i = 0; i < 8; ++i) {
@@ -372,6 +366,15 @@ fft_tc_kernel(const __grid_constant__ CUtensorMap tin, __half *__restrict__ out,
                     }
                     *reinterpret_cast<uint4 *>(o + a0) = make_uint4(v[0], v[1], v[2], v[3]);
                     *reinterpret_cast<uint4 *>(o + g.pitch + a0) = make_uint4(v[4], v[5], v[6], v[7]);
+                } else if (OFF && whole && (a0 < g.pitch || a0 + 8 > kN)) {   // over an end of the plane
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const int a = (a0 + i) & (kN - 1), sh = 16 * (i & 1);
+                        if (a < g.pitch) {
+                            o[a] = __ushort_as_half((unsigned short)(a < g.n_sc ? v[i >> 1] >> sh : 0u));
+                            o[g.pitch + a] = __ushort_as_half((unsigned short)(a < g.n_sc ? v[4 + (i >> 1)] >> sh : 0u));
+                        }
+                    }
                 }
             }
             __syncwarp();
@@ -404,6 +407,7 @@ cudaError_t launch_fft_tc(const Geometry &g, long long rows, const void *in, voi
     if (rows * 64 > 0x7fffffffLL) return cudaErrorInvalidValue;     // TMA row coordinate is 32-bit
     PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
     if (!enc) return cudaErrorNotSupported;
+    FftTcArgs a;
     CUtensorMap map;
     // [rows * 4 s][4 t][4 i][128 mu] FP16: sample j = 16 s + 4 i + t of a row's 64
     cuuint64_t dims[4] = {128, 4, 4, (cuuint64_t)(rows * 4)};
@@ -414,7 +418,9 @@ cudaError_t launch_fft_tc(const Geometry &g, long long rows, const void *in, voi
                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(fft_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+    a.off = (int)((reinterpret_cast<uintptr_t>(out) & 15) / sizeof(__half));
+    auto k = a.off ? fft_tc_kernel<true> : fft_tc_kernel<false>;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);
@@ -423,12 +429,10 @@ cudaError_t launch_fft_tc(const Geometry &g, long long rows, const void *in, voi
     // independent, so a CTA that cannot be resident at once simply runs later.
     long long grid = (long long)sms * (g.fft_cap > 0 && g.fft_cap < kCtasPerSm ? g.fft_cap : kCtasPerSm);
     if (grid > rows) grid = rows;
-    FftTcArgs a;
     a.rows = rows;
     a.n_sc = g.n_sc;
     a.pitch = g.sc_pitch;
-    a.vec = (reinterpret_cast<uintptr_t>(out) & 15) == 0;
-    launch_chained(g.chained, fft_tc_kernel, dim3((unsigned)grid), dim3(kThreads), kSmemBytes, st, map, static_cast<__half *>(out), tw, a, err);
+    launch_chained(g.chained, k, dim3((unsigned)grid), dim3(kThreads), kSmemBytes, st, map, static_cast<__half *>(out), tw, a, err);
     return cudaGetLastError();
 }
 
