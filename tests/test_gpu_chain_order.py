@@ -1,0 +1,97 @@
+"""Kernels that may start before their predecessor ends: calls queued back to back without synchronisation, with the caller's
+own kernels rewriting the inputs in between, and calls replayed from a caller's graph on rewritten inputs give bit for
+bit what synchronised calls give."""
+import pytest
+import torch
+
+from paper_2210_09196_gb300 import binding as B
+from paper_2210_09196_gb300 import denoiser as D
+from paper_2210_09196_gb300 import host, synth
+
+pytestmark = pytest.mark.gpu
+
+CELLS = {
+    "fp32": (synth.SMALL_FP32, B.PUSCH_FORM_FP32, {}),
+    "noise_time": (synth.SMALL_FP32.with_(channel="pdp", beam="dft", doppler_hz=300.0), B.PUSCH_FORM_FP32,
+                   dict(chol_every=4, noise_var=B.PUSCH_NOISE_ESTIMATE)),
+    "deploy": (synth.DEPLOY.with_(n_rx=32, n_sc=600), B.PUSCH_FORM_MIXED, {}),
+    "split": (synth.SMALL_FP32.with_(n_rx=48, n_beams=40, n_sc=301, beam="dft"), B.PUSCH_FORM_FP32, {}),
+}
+
+
+def bits(t):
+    return torch.view_as_real(t) if t.is_complex() else t
+
+
+@pytest.mark.parametrize("name", list(CELLS))
+def test_slots_queued_and_replayed_on_rewritten_inputs(name):
+    cell, form, kw = CELLS[name]
+    slots = synth.make_slots(cell, 3)
+    rx = host.Receiver(host.cfg_for(cell, form, **kw), max_slots=1)
+    ins = [(host.time_tensor([s]), host.pilot_tensor([s])) for s in slots]
+    w = host.beam_tensor(slots[0].W)
+    t, p = (v.clone() for v in ins[0])
+    out = (rx.xhat_buffer(1), rx.bits_buffer(1), rx.status_buffer())
+    want = []
+    for a, b in ins:
+        rx.slot(a, w, b, out)
+        torch.cuda.synchronize()
+        want.append([v.clone() for v in out])
+
+    def check(got):
+        torch.cuda.synchronize()
+        for u, v in zip(got, want):
+            assert all(torch.equal(bits(x), bits(y)) for x, y in zip(u, v))
+
+    got = []
+    for _ in range(4):
+        got = []
+        for a, b in ins:                                  # nothing waits: copies, kernels, copies of the outputs
+            t.copy_(a)
+            p.copy_(b)
+            rx.slot(t, w, p, out)
+            got.append([v.clone() for v in out])
+            for v in out:
+                v.zero_()
+    check(got)
+    s = torch.cuda.Stream()
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=s):
+        rx.slot(t, w, p, out)
+    got = []
+    for a, b in ins:
+        t.copy_(a)
+        p.copy_(b)
+        for v in out:
+            v.zero_()
+        graph.replay()
+        got.append([v.clone() for v in out])
+    check(got)
+    rx.close()
+
+
+def test_learned_estimate_queued_on_rewritten_inputs():
+    cell = synth.DEPLOY.with_(n_rx=16, n_beams=16, n_layers=8, n_fft=1024, n_sc=600, snr_db=20.0)
+    rx = host.Receiver(host.cfg_for(cell), max_slots=1)
+    params = torch.from_numpy(D.init_params(1)).cuda().to(torch.bfloat16)
+    ins = []
+    for s in synth.make_slots(cell, 2):
+        beam = rx.beamform(rx.ofdm_fft(host.time_tensor([s])), host.beam_tensor(s.W)).clone()
+        ins.append((beam, host.pilot_tensor([s])))
+    beam, pil = (v.clone() for v in ins[0])
+    H = rx.H_buffer(1)
+    want = []
+    for a, b in ins:
+        B.pusch_chest_cnn(rx.h, 1, a, b, params, 2.0, H, None, None)
+        torch.cuda.synchronize()
+        want.append(H.clone())
+    for _ in range(4):
+        for (a, b), v in zip(ins, want):
+            beam.copy_(a)
+            pil.copy_(b)
+            B.pusch_chest_cnn(rx.h, 1, beam, pil, params, 2.0, H, None, None)
+            got = H.clone()
+            H.zero_()
+            assert torch.equal(bits(got), bits(v))
+    rx.close()
