@@ -227,10 +227,10 @@ def kernel_of(stage, form, cell=None):
     return k[form] if isinstance(k, dict) else k
 
 
-def measured_traffic(kernel, src, n_slots):
-    """DRAM bytes per launch from the committed ncu summary, scaled to n_slots; None when the kernel's
-    source changed since the capture (the SHA-256 of its source files, in order, is stored beside the
-    counters)."""
+def measured_traffic(kernel, src, n_slots, form=None):
+    """DRAM bytes per launch on the deployment cell from the committed ncu summary, scaled to n_slots; None when the
+    kernel's source changed since the capture (the SHA-256 of its source files, in order, is stored beside the
+    counters) or the capture is of another form (where the kernel's bytes depend on it)."""
     import hashlib
     try:
         with open(os.path.join(ROOT, "profiles", "traffic.json")) as f:
@@ -241,7 +241,7 @@ def measured_traffic(kernel, src, n_slots):
             with open(os.path.join(ROOT, "paper_2210_09196_gb300", "csrc", part), "rb") as f:
                 h.update(f.read())
         sha = h.hexdigest()
-        if sha != e["source_sha256"]:
+        if sha != e["source_sha256"] or (form is not None and e.get("form", form) != form):
             return None
         return int(e["dram_bytes"] / e["slots"] * n_slots)
     except Exception:
@@ -403,7 +403,7 @@ def run_ours(args, rank, world, local):
     dom = max(roof_stages, key=roof_stages.get)
     dom_ms = roof_stages[dom]
     kname, ksrc = kernel_of(dom, form, cell)
-    traffic = measured_traffic(kname, ksrc, n)
+    traffic = measured_traffic(kname, ksrc, n, form) if args.workload == "deploy" else None
     if (dom == "beamform" and kname == "beamform_fp32_kernel") or dom == "detect":
         # FP32 arithmetic, not HBM, bounds these kernels: report them against the derived FP32 ALU peak
         fl = stage_flops(cell, n)[dom]

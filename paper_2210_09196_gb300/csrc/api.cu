@@ -436,8 +436,8 @@ pusch_status run_chain(pusch_handle *h, int s0, int n, size_t freq_off, const vo
     if (ev) cudaEventRecord(ev[2], s);
     const bool est = h->cfg.noise_var == PUSCH_NOISE_ESTIMATE;
     const bool tv = g.chol_every > 0;
-    // the two-symbol-mean table: the estimate itself, or the noise estimator's reference when the estimate
-    // varies in time
+    // the two-symbol-mean table: the estimate where it is constant over the slot. (Where it varies in time nothing reads
+    // this table: the noise estimator takes the observations, and the tables per DMRS symbol replace it below.)
     if ((!tv || est) && (e = pusch::launch_ls_pilots(g, n, beam, pil, ls, s)) != cudaSuccess)
         return cuda_fail(e, "LS pilot table launch");
     if (est && (e = pusch::launch_noise_est(g, n, beam, pil, ne_partial, sigma2, s)) != cudaSuccess)

@@ -33,7 +33,7 @@
 // 16 warps leave 128 registers a thread: with more, the 64 columns of E that an epilogue thread holds spilled, and
 // the spills, missing the little L1 beside 227 KB of shared memory, took 12 k clocks per tile.
 //
-// Measured (GB300, 2 slots of 256 antennas, 64 beams, 3276 subcarriers): 166 us against 671 us on FP32 FMAs; bound by
+// Measured (GB300, 2 slots of 256 antennas, 64 beams, 3276 subcarriers): 162 us against 671 us on FP32 FMAs; bound by
 // the instructions of the warps that load and split (about 900 clocks per stage; HBM needs 440).
 //
 // Every wait is bounded (%globaltimer, 2 s); on expiry the CTA records a timeout in err_word bit 0, all roles
@@ -80,7 +80,7 @@ struct Tf32Shared {
 // range, more). hi stays finite: it is rounded from v brought to the largest magnitude that does not round to infinity,
 // so that values next to FLT_MAX keep theirs in lo, and an infinity or a NaN is in lo alone and gives what it gives in
 // FP32 arithmetic (as hi an infinity would meet both parts of the other operand, whose signs may differ, and its lo were
-// a NaN). The limit is one instruction of some eight per value: 162.5 -> 165.7 us for the case above.
+// a NaN). The limit is one instruction of some eight per value: 157.9 -> 161.7 us for the case above.
 __device__ __forceinline__ void split_tf32(float x, uint32_t &hi, uint32_t &lo) {
     float c;   // x with its magnitude limited
     asm("min.xorsign.abs.f32 %0, %1, %2;" : "=f"(c) : "f"(x), "f"(__uint_as_float(0x7f7fefffu)));

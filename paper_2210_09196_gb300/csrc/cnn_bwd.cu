@@ -26,11 +26,11 @@
 //                    FP32 sums of all products).
 // Two tiles are in flight per CTA (one CTA per SM), 256 threads each. Activations arrive in 2-byte loads along the
 // subcarriers (the caller's layout, any width) and go to shared memory channels-last.
-// Measured (GB300, a step of 1024 grids x 256): out 41, mid 93 each, in 21 us; on FP32 FMAs (weights gradient: one thread
-// per channel pair) the backward pass took 4.0 ms. mid is bound by the chain load - split - products - mask of a tile,
-// of which two overlap (issue 23 %); out and in by the packed FMAs.
-// Every wait is bounded (2 s); after one that expired the loss and the CTA's gradients are NaN, which the layers before take
-// over, the error bit, where there is an error word, is set, and the threads go on without waiting, so all barriers are met: no
+// Measured (GB300, a step of 1024 grids x 256): out 40, mid 93 each, in 20 us; on FP32 FMAs (weights gradient: one thread
+// per channel pair) the backward pass took 4.0 ms. mid is bound by the chain load - split - products - mask - sum of a
+// tile, of which two overlap (issue 28 %, shared-memory pipe 58 %); out and in by the packed FMAs.
+// Every wait is bounded (2 s). After one that expired the loss and the CTA's gradients are NaN, which the layers before take
+// over; the error bit is set where there is an error word; the threads go on without waiting, so all barriers are met: no
 // address depends on what a wait was for. MMAs in flight are drained (bounded) before TMEM is freed, on a barrier of its
 // own: those of the products may be a phase behind by then.
 #include "tc_common.cuh"

@@ -27,10 +27,10 @@
 // Measured (GB300, 512 grids of 3276 subcarriers): 190 us, 460 TFLOP/s of the network's arithmetic; layer by layer through
 // HBM, with layers 1 and 4 on FP32 FMAs, the same took 780 us. Bound by the threads' share: per tile about 10 k clocks of
 // packed FMAs (layer 1), 5 k of bias, ReLU and packing, 6 k of waiting for products, four tiles overlapping.
-// Every wait is bounded (2 s); after one that expired the threads go on without waiting (the CTA's outputs from then on are
-// NaN and the error bit, where the caller has an error word, is set), so all barriers are met: no address depends on what a wait was for. MMAs in flight are drained
-// (bounded) before TMEM is freed, on a barrier of its own: that of the products may be a phase behind by then, and a wait
-// for its newest phase would pass at once.
+// Every wait is bounded (2 s). After one that expired the CTA's outputs are NaN, the error bit is set where the caller has an
+// error word, and the threads go on without waiting, so all barriers are met: no address depends on what a wait was for.
+// MMAs in flight are drained (bounded) before TMEM is freed, on a barrier of its own: that of the products may be a phase
+// behind by then, and a wait for its newest phase would pass at once.
 #include "tc_common.cuh"
 
 namespace pusch {

@@ -25,16 +25,17 @@
 //     mod 4096, octet e = t + 4 half. The remainder hr = (n_sc / 2 + off) mod 8, off the output's distance from a
 //     16-byte boundary in values, rotates k0; only octet 0 then mixes two k1, and its first hr elements come from the
 //     lanes of k1 - 1 (eight exchanges per 64 x 8 block). Where off > 0, the octets over a plane's ends are stored
-//     value by value (7,168 rows into a plane 2, 4 or 8 bytes off a boundary: 187, 194 and 205 us when all values were
-//     stored singly, aligned 59.6).
+//     value by value (7,168 rows into a plane 2, 4 or 8 bytes off a boundary: 70 us at most; 187, 194 and 205 us when all
+//     of its values were stored singly).
 // A 4096-point transform thus costs two MMA passes (8 MMAs of 128 x 128 x 16) and one pass of twiddles and
 // transposition through shared memory.
 //
 // What bounds it: the reading warps. With the data as the MMA's A operand (a complex value's sums in two lanes) the
 // LSU pipe was 67 % and issue 57 % busy: 128 lane exchanges and 51 2-byte stores per row and warp, 70.6 us for 7,168
-// rows with 3276 of 4096 bins kept. Here 16 exchanges and 8 16-byte stores per row: 58.6 us (52 % of the measured copy
-// rate), of which the accumulator reads are the largest part of the LSU pipe's work (1,024 of its wavefronts
-// per row). Three CTAs per SM, also with a two-stage ring: 58.7 and 60.1 us; octet 0 stored one element at a time 108 us.
+// rows with 3276 of 4096 bins kept. Here 16 exchanges and 8 16-byte stores per row: 56.2 us (55 % of the measured copy
+// rate), of which the accumulator reads are the largest part of the LSU pipe's work (1,024 of its wavefronts per row).
+// Measured while unaligned outputs had a path in the same kernel, 58.6 us then: three CTAs per SM, also with a two-stage
+// ring, 58.7 and 60.1 us; octet 0 stored one element at a time 108 us.
 //
 // Roles (persistent CTAs, four per SM, 128 TMEM columns each): warps 0-3 read the accumulators (warp q owns TMEM
 // lane quarter q) and write the next operand or the output; warp 4 issues the row copies (TMA, a one-stage ring)
@@ -61,7 +62,7 @@ constexpr int kTmemCols = 128;
 constexpr int kStages = 1;
 
 constexpr uint32_t kRowBytes = kN * 4;                      // one row of FP16 complex samples: 16 KB
-constexpr uint32_t kOffIn = 0;                              // input ring (stage-1 A operands, 1024-aligned)
+constexpr uint32_t kOffIn = 0;                              // input ring (stage-1 B operands, 1024-aligned)
 constexpr uint32_t kOffA = kOffIn + kStages * kRowBytes;    // A: [128][64] FP16, K-major, 16 KB
 constexpr uint32_t kOffY = kOffA + 16384;                   // Y: stage 2's B operand [128][64] FP16, K-major
 constexpr uint32_t kLboY = 144, kSboY = 1184;               // 8 core matrices of 128 B (+ 16), 16 column groups (+ 32)
@@ -209,7 +210,7 @@ fft_tc_kernel(const __grid_constant__ CUtensorMap tin, __half *__restrict__ out,
             const uint32_t idesc = idesc_f16(128, 128, false, true);    // stage 1: B (the row) N-major
             const uint32_t idesc2 = idesc_f16(128, 128, false, false);
             // the time samples are read once: evict-first, so that they do not push the FFT output (the next
-            // kernel's input) out of L2 (an evict-last hint on the 2-byte output stores measured slower)
+            // kernel's input) out of L2
             const uint64_t pol_in = l2_policy_evict_first();
             auto issue = [&](long long i) {
                 const int s = (int)(i % kStages);
