@@ -15,7 +15,7 @@ CELLS = {
     "noise_time": (synth.SMALL_FP32.with_(channel="pdp", beam="dft", doppler_hz=300.0), B.PUSCH_FORM_FP32,
                    dict(chol_every=4, noise_var=B.PUSCH_NOISE_ESTIMATE)),
     "deploy": (synth.DEPLOY.with_(n_rx=32, n_sc=600), B.PUSCH_FORM_MIXED, {}),
-    "split": (synth.SMALL_FP32.with_(n_rx=48, n_beams=40, n_sc=301, beam="dft"), B.PUSCH_FORM_FP32, {}),
+    "split": (synth.SMALL_FP32.with_(n_rx=80, n_beams=40, n_sc=301, beam="dft"), B.PUSCH_FORM_FP32, {}),
 }
 
 
