@@ -631,15 +631,12 @@ pusch_status pusch_slot_host(pusch_handle *h, int n_slots, const void *time_in_h
     const pusch::Geometry &g = h->geo;
     cudaError_t e;
     if (!h->h_time) {  // staging buffers, sized for max_slots, allocated on first use
-        if ((e = cudaMalloc(&h->h_time, time_bytes(g, h->max_slots))) != cudaSuccess) return cuda_fail(e, "staging");
-        if ((e = cudaMalloc((void **)&h->h_pilots, pilot_bytes(g, h->max_slots))) != cudaSuccess)
-            return cuda_fail(e, "staging");
-        if ((e = cudaMalloc((void **)&h->h_xhat, xhat_count(g, h->max_slots) * sizeof(float2))) != cudaSuccess)
-            return cuda_fail(e, "staging");
-        if ((e = cudaMalloc((void **)&h->h_bits, xhat_count(g, h->max_slots))) != cudaSuccess)
-            return cuda_fail(e, "staging");
-        if ((e = cudaMalloc((void **)&h->h_status, 4 * sizeof(uint32_t))) != cudaSuccess)
-            return cuda_fail(e, "staging");
+        e = pusch::malloc_all({{&h->h_time, time_bytes(g, h->max_slots)},
+                               {(void **)&h->h_pilots, pilot_bytes(g, h->max_slots)},
+                               {(void **)&h->h_xhat, xhat_count(g, h->max_slots) * sizeof(float2)},
+                               {(void **)&h->h_bits, xhat_count(g, h->max_slots)},
+                               {(void **)&h->h_status, 4 * sizeof(uint32_t)}});
+        if (e != cudaSuccess) return cuda_fail(e, "staging");
     }
     cudaStream_t s = (cudaStream_t)stream;
     st = slot_batch(h, n_slots, h->h_time, W, h->h_pilots, h->h_xhat, h->h_bits, h->h_status, s, time_in_host,

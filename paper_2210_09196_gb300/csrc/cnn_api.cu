@@ -114,10 +114,10 @@ pusch_status pusch_chest_cnn(pusch_handle *h, int n_slots, const void *beam, con
     cudaError_t e;
     if (!h->cnn_grid) {  // workspace sized for max_slots, allocated on first use
         const size_t px = (size_t)grids_max * 2 * g.n_sc;
-        if ((e = cudaMalloc(&h->cnn_grid, px * 2 * sizeof(__nv_bfloat16))) != cudaSuccess ||
-            (e = cudaMalloc((void **)&h->cnn_scale, (size_t)grids_max * sizeof(float))) != cudaSuccess ||
-            (e = cudaMalloc((void **)&h->cnn_y, px * 2 * sizeof(float))) != cudaSuccess)
-            return cfail(PUSCH_ERR_CUDA, "CNN workspace allocation", e);
+        e = pusch::malloc_all({{&h->cnn_grid, px * 2 * sizeof(__nv_bfloat16)},
+                               {(void **)&h->cnn_scale, (size_t)grids_max * sizeof(float)},
+                               {(void **)&h->cnn_y, px * 2 * sizeof(float)}});
+        if (e != cudaSuccess) return cfail(PUSCH_ERR_CUDA, "CNN workspace allocation", e);
     }
     cudaStream_t s = (cudaStream_t)stream;
     const int grids = n_slots * g.n_layers * g.n_beams;

@@ -8,6 +8,7 @@
 
 #include <cuda_bf16.h>
 
+#include <initializer_list>
 #include <vector>
 
 #include "../../include/pusch.h"
@@ -86,6 +87,27 @@ inline cudaError_t launch_chained(bool chained, void (*k)(P...), dim3 grid, dim3
                                   A... args) {
     const ChainedConfig c(chained, grid, block, smem, st);
     return cudaLaunchKernelEx(&c.cfg, k, static_cast<P>(args)...);
+}
+
+// Device buffers that belong together: all of them, or none (the pointers are NULL again and the error is not left behind
+// for the next check of a launch), so that a call that failed for want of memory can be made again.
+struct DeviceBuffer {
+    void **p;
+    size_t bytes;
+};
+inline cudaError_t malloc_all(std::initializer_list<DeviceBuffer> all) {
+    for (const DeviceBuffer &b : all) {
+        const cudaError_t e = cudaMalloc(b.p, b.bytes);
+        if (e == cudaSuccess) continue;
+        *b.p = nullptr;
+        for (const DeviceBuffer &c : all) {
+            cudaFree(*c.p);
+            *c.p = nullptr;
+        }
+        cudaGetLastError();
+        return e;
+    }
+    return cudaSuccess;
 }
 
 // ---------------------------------------------------------------------------------- derived geometry
